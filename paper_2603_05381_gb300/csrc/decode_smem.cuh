@@ -260,10 +260,13 @@ struct Regs<float, N> {
     }
 };
 
-// 1 if lambda > 0, else 0 (NaN and -0 give 0), on the FMA pipe: saturate(lambda x 2^64).
-// A positive lambda below 2^-64 would give a fraction; such a lambda is a tie by any margin
-// the decoder distinguishes.
-__device__ __forceinline__ float keep_f(float lam) { return __saturatef(__fmul_rn(lam, 0x1p64f)); }
+// min(u, 1) for u >= 0 (saturate), on the FMA pipe: the leave-one-out sum takes the row's
+// maximum, 2^(m1 - m2) >= 1, as 1.
+__device__ __forceinline__ float sat1(float u) {
+    float r;
+    asm("add.sat.f32 %0, %1, 0f00000000;" : "=f"(r) : "f"(u));
+    return r;
+}
 
 __device__ __forceinline__ float max3f(float a, float b, float c) {
     float r;
@@ -292,12 +295,20 @@ __host__ __device__ constexpr int blocks_for(int nt, int elem_bytes, int msg_byt
     return (elem_bytes == 4 && (nt == 384 || nt == 448 || (nt == 512 && msg_bytes == 2))) ? 2 : min_blocks(nt);
 }
 
-// REG = true keeps each thread's own outputs M[i][k] in registers between iterations (no
-// strided shared-memory read per message); REG = false reads them back from Mt[k][i].
+// Rows watched for the convergence decision (FP32 arithmetic): a shot has converged only if
+// every row keeps exactly one variable, so one row that does not settles an iteration's
+// decision.  kWatch warps each look at one row that was seen violating; only when all of them
+// have stopped violating is every row counted.  Counting every row in every iteration took an
+// add, a multiply and an own-output read per message, or a register copy of the outputs (24
+// warp instructions per 32 updates at 144 rows, 19 without); measured on 200,001 d = 21
+// code-capacity shots 99.9 -> 88.2 ms, 300,000 d = 13 circuit shots 281.4 -> 269.0 ms, 10^6
+// d = 9 code-capacity shots 16.0 -> 14.3 ms, outputs equal.
+constexpr int kWatch = 4;
+
 // RW = true: the B-BP4MF second stage.  The shot's priors, pair weights and parities are
 // computed in the block by Dijkstra from every defect over per-qubit weights derived from
 // the first stage's posteriors (instead of being gathered from the static tables).
-template <typename T, int CH, int G, bool TRACE, bool REG, bool RW = false, typename MS = T>
+template <typename T, int CH, int G, bool TRACE, bool RW = false, typename MS = T>
 __global__ void __launch_bounds__(CH * G * G, blocks_for(CH * G * G, (int)sizeof(T), (int)sizeof(MS))) decode_smem_kernel(const DecodeArgs a) {
     constexpr int SMAX = CH * G;
     constexpr int NT = SMAX * G;
@@ -334,6 +345,7 @@ __global__ void __launch_bounds__(CH * G * G, blocks_for(CH * G * G, (int)sizeof
     unsigned char* rw_par = rw_done + (NT / 32) * rw_nodes;
     __shared__ int sh_item, sh_s, sh_best_par, sh_best_forced, sh_improve, sh_use_best;
     __shared__ double sh_best_w;
+    __shared__ unsigned sh_bad[NT / 32];  // full count: each warp's rows that do not keep exactly one
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int i = warp * R + (lane % R);   // row (factor) of this thread
@@ -548,102 +560,68 @@ __global__ void __launch_bounds__(CH * G * G, blocks_for(CH * G * G, (int)sizeof
         // skips the read and compute phases (it still takes part in every barrier)
         const bool wact = warp * R < s;
         Regs<T, CH> q;
-        Regs<T, REG ? CH : 2> mo;
-        int am_prev = -1;          // REG: argmax column of the previous update and its output
-        T out_am = T(0);
-        T out_am_gen = T(0);       // REG, FP32: the generic formula's value held in registers for it
+        constexpr int NWATCH = NT / 32 < kWatch ? NT / 32 : kWatch;
+        int watch = warp < NWATCH ? warp * s / NWATCH : 0;  // this warp's watched row
         int t = 0;
         bool any_conv = false, forced_ran = false;
         int out_par = 0, out_forced = 0, out_from_best = 0;
         int partner = -1;
 
         for (;;) {
-            // ---- read phase: Q = l + M[k][i]/alpha for the next update; for t > 0 the
-            // marginalization of lambda^t = l + (M[i][k] + M[k][i]).  FP32: the row's
-            // maximum / second maximum scan of the next update runs in the same loop (it needs
-            // only Q), so that the shared-memory loads and the scan's ALU work overlap; the
-            // scan is over columns in the same order as a separate pass, so its result is the
-            // same
+            // ---- read phase: Q = l + M[k][i]/alpha for the next update.  FP32: the row's maximum /
+            // second maximum scan of the next update runs in the same loop (it needs only Q), so
+            // that the shared-memory loads and the scan's ALU work overlap.  The marginalization of
+            // lambda^t = l + (M[i][k] + M[k][i]) (t > 0) is not evaluated here: see the watched rows
+            // below.
             Mask bits = 0;
-            float cntf = 0.f;
             float sa1 = Num<float>::ninf(), sa2 = Num<float>::ninf();
-            int sac = 0x7fffffff;
-            auto scan_pair = [&](int j, float v, float w) {
-                // (max, second max, column) of the pairs so far; ties to the smaller column
-                const float hi = fmaxf(v, w), lo = fminf(v, w);
-                const int ih = v >= w ? 2 * j : 2 * j + 1;
-                const bool gt = hi > sa1;
+            int sab = 0;
+            // (max, second max, first block of the max) over the blocks of four columns so far.
+            // Only the block of four is tracked (one compare and one select for four columns
+            // instead of two per column: the compare, select and max instructions bound this
+            // phase); the thread that holds the row's maximum finds the column in its block
+            // afterwards.
+            auto scan4 = [&](int b, float2 p0, float2 p1) {
+                const float h0 = fmaxf(p0.x, p0.y), l0 = fminf(p0.x, p0.y);
+                const float h1 = fmaxf(p1.x, p1.y), l1 = fminf(p1.x, p1.y);
+                const float hi = fmaxf(h0, h1), lo = max3f(l0, l1, fminf(h0, h1));
+                sab = hi > sa1 ? b : sab;
                 sa2 = max3f(sa2, lo, fminf(sa1, hi));
                 sa1 = fmaxf(sa1, hi);
-                sac = gt ? ih : sac;
             };
             if (!wact) {
             } else if (!act) {
 #pragma unroll
                 for (int c = 0; c < CH; ++c) q[c] = ninf;
+            } else if constexpr (std::is_same<T, float>::value) {
+                const float2 ainv2 = make_float2(ainv, ainv);
+#pragma unroll
+                for (int j = 0; j < CH / 2; j += 2) {
+                    q.p[j] = __ffma2_rn(RM2(j), ainv2, RL2(j));
+                    q.p[j + 1] = __ffma2_rn(RM2(j + 1), ainv2, RL2(j + 1));
+                    scan4(j / 2, q.p[j], q.p[j + 1]);
+                }
+                if (TRACE && tr_on && trl && t > 0) {
+#pragma unroll
+                    for (int c = 0; c < CH; ++c) {
+                        const int k = COL(c);
+                        if (k < s)
+                            trl[((size_t)shot * a.s_cap + i) * a.s_cap + k] =
+                                (k == i ? RL(c) + Dg[i] : RL(c) + (CM(c) + RM(c))) * (float)kLn2;
+                    }
+                }
             } else {
                 if (t == 0) {
-                    if constexpr (std::is_same<T, float>::value) {
-                        const float2 ainv2 = make_float2(ainv, ainv);
 #pragma unroll
-                        for (int j = 0; j < CH / 2; ++j) {
-                            q.p[j] = __ffma2_rn(RM2(j), ainv2, RL2(j));
-                            scan_pair(j, q.p[j].x, q.p[j].y);
-                        }
-                    } else {
-#pragma unroll
-                        for (int c = 0; c < CH; ++c) q[c] = B2<T>::fma_(RM(c), ainv, RL(c));
-                    }
-                } else if constexpr (std::is_same<T, float>::value) {
-                    // two columns per packed instruction; same roundings as the scalar form.
-                    // The kept count is a sum of keep(lambda) in {0, 1} on the FMA pipe; the
-                    // kept column itself is found only when every row has exactly one
-                    // (row_kept_column below).
-                    const float2 ainv2 = make_float2(ainv, ainv);
-                    float2 cnt2 = make_float2(0.f, 0.f);
-#pragma unroll
-                    for (int j = 0; j < CH / 2; ++j) {
-                        const int c = 2 * j;
-                        const float2 l = RL2(j);
-                        const float2 x = RM2(j);
-                        float2 own;
-                        if constexpr (REG)
-                            own = mo.p[j];
-                        else
-                            own = make_float2(CM(c), CM(c + 1));
-                        q.p[j] = __ffma2_rn(x, ainv2, l);
-                        scan_pair(j, q.p[j].x, q.p[j].y);
-                        const float2 lam = __fadd2_rn(l, __fadd2_rn(own, x));
-                        cnt2 = __fadd2_rn(cnt2, make_float2(keep_f(lam.x), keep_f(lam.y)));
-                        if (tr_on && trl && COL(c) < s)
-                            trl[((size_t)shot * a.s_cap + i) * a.s_cap + COL(c)] = lam.x * (float)kLn2;
-                        if (tr_on && trl && COL(c + 1) < s)
-                            trl[((size_t)shot * a.s_cap + i) * a.s_cap + COL(c + 1)] = lam.y * (float)kLn2;
-                    }
-                    cntf = cnt2.x + cnt2.y;
-                    if (!REG && own_diag) {
-                        // the generic term used Mt[i][i] = 0 on both sides: lambda_ii = l_ii
-                        const float lii = Lm[i * P + i];
-                        const float lam = lii + Dg[i];
-                        cntf += keep_f(lam) - keep_f(lii + (0.f + 0.f));
-                        if (tr_on && trl) trl[((size_t)shot * a.s_cap + i) * a.s_cap + i] = lam * (float)kLn2;
-                    }
-                    if (REG && owner_of<PAIR, G>(am_prev) == g) {
-                        // the register copy of the argmax column holds the generic output
-                        const float l = Lm[i * P + am_prev], x = m_ld1(Mt + i * PM + am_prev, am_prev);
-                        const float lam = l + (out_am + x);
-                        cntf += keep_f(lam) - keep_f(l + (out_am_gen + x));
-                        if (tr_on && trl) trl[((size_t)shot * a.s_cap + i) * a.s_cap + am_prev] = lam * (float)kLn2;
-                    }
+                    for (int c = 0; c < CH; ++c) q[c] = B2<T>::fma_(RM(c), ainv, RL(c));
                 } else {
                     Mask b0 = 0, b1 = 0;
 #pragma unroll
                     for (int c = 0; c < CH; ++c) {
                         const T l = RL(c);
                         const T x = RM(c);
-                        const T own = REG ? mo[REG ? c : 0] : CM(c);
                         q[c] = B2<T>::fma_(x, ainv, l);
-                        const T lam = l + (own + x);
+                        const T lam = l + (CM(c) + x);
                         if (c & 1)
                             b1 |= (Mask)(lam > T(0) ? 1u : 0u) << c;
                         else
@@ -652,43 +630,96 @@ __global__ void __launch_bounds__(CH * G * G, blocks_for(CH * G * G, (int)sizeof
                             trl[((size_t)shot * a.s_cap + i) * a.s_cap + COL(c)] = lam * (T)kLn2;
                     }
                     bits = b0 | b1;
-                    if (!REG && own_diag) {
+                    if (own_diag) {
                         // the boundary variable v_ii: lambda_ii = l_ii + M[i][i]
                         const T lam = Lm[i * P + i] + Dg[i];
                         bits = (bits & ~((Mask)1 << c_diag)) | ((Mask)(lam > T(0) ? 1u : 0u) << c_diag);
                         if (tr_on && trl) trl[((size_t)shot * a.s_cap + i) * a.s_cap + i] = lam * (T)kLn2;
                     }
-                    if (REG && owner_of<PAIR, G>(am_prev) == g) {
-                        // the argmax column's own output is out_am, not the generic formula's
-                        const int ca = reg_of<PAIR, G>(am_prev);
-                        const T lam = Lm[i * P + am_prev] + (out_am + m_ld1(Mt + i * PM + am_prev, am_prev));
-                        bits = (bits & ~((Mask)1 << ca)) | ((Mask)(lam > T(0) ? 1u : 0u) << ca);
-                        if (tr_on && trl) trl[((size_t)shot * a.s_cap + i) * a.s_cap + am_prev] = lam * (T)kLn2;
-                    }
                 }
             }
-            // FP32: the row's (m1, m2, argmax column) of the next update, over the G threads
+            // FP32: the row's (m1, m2) of the next update over the G threads, and the column of m1
+            // in the thread that holds it (own_max).  No index travels with the maxima: where
+            // m1 > m2 exactly one thread holds m1, and where m1 == m2 the generic output formula and
+            // the one for the maximum's column give the same value (2^(m2 - m1) = 1, and S - 1 is
+            // exact), so any holder may write it.
             T m1 = ninf, m2 = ninf;
             int am = 0x7fffffff;
+            bool own_max = false;
+            int conv, chosen = -1;
             if constexpr (std::is_same<T, float>::value) {
                 if (wact) {
                     m1 = sa1;
                     m2 = sa2;
-                    am = sac < CH ? COL(sac) : 0x7fffffff;
 #pragma unroll
                     for (int off = R; off < 32; off <<= 1) {
                         const T o1 = __shfl_xor_sync(kFull, m1, off);
                         const T o2 = __shfl_xor_sync(kFull, m2, off);
-                        const int ok = __shfl_xor_sync(kFull, am, off);
-                        combine_max(m1, m2, am, o1, o2, ok);
+                        m2 = max3f(m2, o2, fminf(m1, o1));
+                        m1 = fmaxf(m1, o1);
+                    }
+                    own_max = act && sa1 == m1;
+                    if (own_max) {
+                        // the same values as in the loop above: Mt is still as it was read
+                        const float2 ainv2 = make_float2(ainv, ainv);
+                        const float2 p0 = __ffma2_rn(m_ld2(row_m + 4 * G * sab, k0 + 4 * G * sab), ainv2,
+                                                     *reinterpret_cast<const float2*>(row_l + 4 * G * sab));
+                        const float p1x = __fmaf_rn(m_ld1(row_m + 4 * G * sab + 2 * G, k0 + 4 * G * sab + 2 * G), ainv,
+                                                    row_l[4 * G * sab + 2 * G]);
+                        am = k0 + 4 * G * sab + (p0.x == m1 ? 0 : p0.y == m1 ? 1 : p1x == m1 ? 2 * G : 2 * G + 1);
                     }
                 }
-            }
-            int cnt, chosen = -1;
-            if constexpr (std::is_same<T, float>::value) {
+                // ---- convergence of lambda^t.  The watched rows are counted by one warp each; a
+                // single row that does not keep exactly one variable settles the vote (one reader
+                // warp per row costs a few tens of instructions, counting every row an add, a
+                // compare and two shared-memory reads per message).  In a d = 13 circuit shot 20
+                // rows violate in the median iteration, so the full count runs in about 1% of them
+                // besides the ones that converge.
+                int violated = t == 0;
+                if (t > 0 && warp < NWATCH) {
+                    const int r = watch;
+                    int cnt = 0;
 #pragma unroll
-                for (int off = R; off < 32; off <<= 1) cntf += __shfl_xor_sync(kFull, cntf, off);
-                cnt = (int)cntf;
+                    for (int k = lane; k < SMAX; k += 32) {
+                        const float l = Lm[r * P + k];
+                        const float lam = k == r ? l + Dg[r] : l + (m_ld1(Mt + k * PM + r, r) + m_ld1(Mt + r * PM + k, k));
+                        cnt += lam > 0.f ? 1 : 0;
+                    }
+                    violated = __reduce_add_sync(kFull, cnt) != 1;
+                    if (!violated) watch = r + 1 < s ? r + 1 : 0;
+                }
+                // (also the barrier between reading Mt and overwriting it)
+                conv = !__syncthreads_or(violated);
+                if (conv) {
+                    // no watched row violates: count every row, and find its kept column
+                    int k1 = -1, cnt = 0;
+                    if (act) {
+#pragma unroll
+                        for (int c = 0; c < CH; ++c) {
+                            const int k = COL(c);
+                            const float l = RL(c);
+                            const float lam = k == i ? l + Dg[i] : l + (CM(c) + RM(c));
+                            cnt += lam > 0.f ? 1 : 0;
+                            if (lam > 0.f) k1 = k;
+                        }
+                    }
+#pragma unroll
+                    for (int off = R; off < 32; off <<= 1) {
+                        cnt += __shfl_xor_sync(kFull, cnt, off);
+                        k1 = max(k1, __shfl_xor_sync(kFull, k1, off));
+                    }
+                    chosen = k1;
+                    const bool bad = act && cnt != 1;
+                    const unsigned badrows = __ballot_sync(kFull, bad) & (R == 32 ? kFull : (1u << (R & 31)) - 1u);
+                    if (lane == 0) sh_bad[warp] = badrows;
+                    conv = __syncthreads_and(!bad);
+                    if (!conv && warp < NWATCH) {
+                        // watch the first violating row at or after this warp's share of the rows
+                        int w = warp * (NT / 32) / NWATCH;
+                        while (sh_bad[w] == 0u) w = w + 1 < NT / 32 ? w + 1 : 0;
+                        watch = w * R + __ffs((int)sh_bad[w]) - 1;
+                    }
+                }
             } else {
                 // kept count << 16 plus (first kept column + 1), summed over the row's G threads:
                 // the count is exact, the column is the row's only kept one when the count is 1
@@ -696,41 +727,9 @@ __global__ void __launch_bounds__(CH * G * G, blocks_for(CH * G * G, (int)sizeof
                          (bits ? COL((sizeof(Mask) == 8 ? __ffsll((long long)bits) : __ffs((int)bits)) - 1) + 1 : 0);
 #pragma unroll
                 for (int off = R; off < 32; off <<= 1) pk += __shfl_xor_sync(kFull, pk, off);
-                cnt = pk >> 16;
+                const int cnt = pk >> 16;
                 chosen = (pk & 0xFFFF) - 1;
-            }
-            const int conv = __syncthreads_and(t > 0 && (!act || cnt == 1));
-            if constexpr (std::is_same<T, float>::value) {
-                if (conv && wact) {
-                    // every row keeps exactly one variable: find it (the same lambdas as above)
-                    int k1 = -1;
-                    if (act) {
-#pragma unroll
-                        for (int j = 0; j < CH / 2; ++j) {
-                            const int c = 2 * j;
-                            const float2 l = RL2(j);
-                            const float2 x = RM2(j);
-                            float2 own;
-                            if constexpr (REG)
-                                own = mo.p[j];
-                            else
-                                own = make_float2(CM(c), CM(c + 1));
-                            float2 lam = __fadd2_rn(l, __fadd2_rn(own, x));
-                            if (!REG && own_diag && c == c_diag) lam.x = Lm[i * P + i] + Dg[i];
-                            if (!REG && own_diag && c + 1 == c_diag) lam.y = Lm[i * P + i] + Dg[i];
-                            if (REG && owner_of<PAIR, G>(am_prev) == g) {
-                                const float fix = Lm[i * P + am_prev] + (out_am + m_ld1(Mt + i * PM + am_prev, am_prev));
-                                if (c == reg_of<PAIR, G>(am_prev)) lam.x = fix;
-                                if (c + 1 == reg_of<PAIR, G>(am_prev)) lam.y = fix;
-                            }
-                            if (lam.x > 0.f) k1 = COL(c);
-                            if (lam.y > 0.f) k1 = COL(c + 1);
-                        }
-                    }
-#pragma unroll
-                    for (int off = R; off < 32; off <<= 1) k1 = max(k1, __shfl_xor_sync(kFull, k1, off));
-                    chosen = k1;
-                }
+                conv = __syncthreads_and(t > 0 && (!act || cnt == 1));
             }
 
             if (t > 0) {
@@ -745,7 +744,7 @@ __global__ void __launch_bounds__(CH * G * G, blocks_for(CH * G * G, (int)sizeof
                     forced_ran = true;
                     if (act && g == 0) matched[i] = 0;
                     __syncthreads();
-                    const T lii = act ? (REG ? Lm[i * P + i] + (mo.get(c_diag) + T(0)) : Lm[i * P + i] + Dg[i]) : ninf;
+                    const T lii = act ? Lm[i * P + i] + Dg[i] : ninf;
                     if (a.forced_static) {
                         // the paper's static partition: row i's block is v_ik, k >= i; its
                         // maximum (ties: smaller k) represents factor i; representatives are
@@ -757,10 +756,7 @@ __global__ void __launch_bounds__(CH * G * G, blocks_for(CH * G * G, (int)sizeof
                             for (int c = 0; c < CH; ++c) {
                                 const int k = COL(c);
                                 if (k >= i && k < s) {
-                                    const T own = REG ? mo[REG ? c : 0] : CM(c);
-                                    T lam = RL(c) + (own + RM(c));
-                                    if (!REG && k == i) lam = lii;
-                                    if (REG && k == am_prev) lam = RL(c) + (out_am + RM(c));
+                                    const T lam = k == i ? lii : RL(c) + (CM(c) + RM(c));
                                     if (bk < 0 || lam > bl) {
                                         bl = lam;
                                         bk = k;
@@ -820,10 +816,7 @@ __global__ void __launch_bounds__(CH * G * G, blocks_for(CH * G * G, (int)sizeof
                             for (int c = 0; c < CH; ++c) {
                                 const int k = COL(c);
                                 if (k == i || !matched[k]) {
-                                    const T own = REG ? mo[REG ? c : 0] : CM(c);
-                                    T lam = RL(c) + (own + RM(c));
-                                    if (!REG && k == i) lam = lii;
-                                    if (REG && k == am_prev) lam = RL(c) + (out_am + RM(c));
+                                    const T lam = k == i ? lii : RL(c) + (CM(c) + RM(c));
                                     if (bk < 0 || lam > bl) {
                                         bl = lam;
                                         bk = k;
@@ -934,10 +927,10 @@ __global__ void __launch_bounds__(CH * G * G, blocks_for(CH * G * G, (int)sizeof
                     float2 s2 = make_float2(0.f, 0.f);
 #pragma unroll
                     for (int j = 0; j < CH / 2; ++j) {
-                        const float2 dq = __fadd2_rn(make_float2(fminf(q.p[j].x, m2), fminf(q.p[j].y, m2)), nm2);
+                        const float2 dq = __fadd2_rn(q.p[j], nm2);
                         const float2 u = make_float2(B2<float>::ex2(dq.x), B2<float>::ex2(dq.y));
                         q.p[j] = u;
-                        s2 = __fadd2_rn(s2, u);
+                        s2 = __fadd2_rn(s2, make_float2(sat1(u.x), sat1(u.y)));
                     }
                     float S32 = s2.x + s2.y;
 #pragma unroll
@@ -963,44 +956,31 @@ __global__ void __launch_bounds__(CH * G * G, blocks_for(CH * G * G, (int)sizeof
                             const float2 lg = make_float2(B2<float>::lg2(y.x), B2<float>::lg2(y.y));
                             const float2 out = __ffma2_rn(lg, neg1, nm1);
                             if constexpr (HALF) {
-                                // store the rounded pair (relative to r_i); the register copy is
-                                // the stored value decoded as every reader decodes it, so that
-                                // both ends of a variable see the same message
+                                // store the rounded pair (relative to r_i): both ends of a variable
+                                // read the same message
                                 const unsigned pk2 = IO::pack(out.x, out.y);
                                 *reinterpret_cast<unsigned short*>(CMP(2 * j)) = (unsigned short)(pk2 & 0xFFFFu);
                                 *reinterpret_cast<unsigned short*>(CMP(2 * j + 1)) = (unsigned short)(pk2 >> 16);
-                                if constexpr (REG) mo.p[j] = __fadd2_rn(IO::unpack(pk2), make_float2(-rf, -rf));
                             } else {
                                 *CMP(2 * j) = out.x;
                                 *CMP(2 * j + 1) = out.y;
-                                if constexpr (REG) mo.p[j] = out;
                             }
                         }
-                        float oam = -m2 - B2<float>::lg2(S32 - 1.f);
-                        if constexpr (HALF) {
-                            const float st_am = __fmaf_rn(B2<float>::lg2(S32 - 1.f), -1.f, rf - m2);
-                            if (owner_of<PAIR, G>(am) == g) IO::st(Mt + am * PM + i, st_am);
-                            oam = IO::unpack(IO::pack(st_am, 0.f)).x + (-rf);
-                        } else if (owner_of<PAIR, G>(am) == g) {
-                            IO::st(Mt + am * PM + i, oam);
-                        }
-                        if (REG) {
-                            am_prev = am;
-                            out_am = oam;
-                            // what the packed output loop produced for the argmax column: u = ex2(0)
-                            const float u0 = B2<float>::ex2(0.f);
-                            float og = __fmaf_rn(B2<float>::lg2(__fmaf_rn(-cf32, u0, Aa32)), -1.f, HALF ? dref32 : -m1);
-                            if constexpr (HALF) og = IO::unpack(IO::pack(og, 0.f)).x + (-rf);
-                            out_am_gen = og;
+                        if (own_max) {
+                            const float lgS = B2<float>::lg2(S32 - 1.f);
+                            if constexpr (HALF)
+                                IO::st(Mt + am * PM + i, __fmaf_rn(lgS, -1.f, rf - m2));
+                            else
+                                IO::st(Mt + am * PM + i, -m2 - lgS);
                         }
                         if (own_diag) {
                             if constexpr (HALF) {
                                 // the diagonal holds r_i, which decodes to exactly 0
-                                if (!REG) Dg[i] = IO::ld(Mt + i * PM + i) + (-rf);
+                                Dg[i] = IO::ld(Mt + i * PM + i) + (-rf);
                                 IO::st(Mt + i * PM + i, rf);
                                 nrefv[i] = -rf;
                             } else {
-                                if (!REG) Dg[i] = IO::ld(Mt + i * PM + i);
+                                Dg[i] = IO::ld(Mt + i * PM + i);
                                 Mt[i * PM + i] = MS(0.f);
                             }
                         }
@@ -1061,16 +1041,11 @@ __global__ void __launch_bounds__(CH * G * G, blocks_for(CH * G * G, (int)sizeof
                         for (int c = 0; c < CH; ++c) {
                             const T out = -m1 - B2<T>::lg2(B2<T>::fma_(-cf, q[c], Aa));
                             *CMP(c) = out;
-                            if (REG) mo[REG ? c : 0] = out;
                         }
                         const T oam = -m2 - B2<T>::lg2(S - T(1));
                         if (owner_of<PAIR, G>(am) == g) IO::st(Mt + am * PM + i, oam);
-                        if (REG) {
-                            am_prev = am;
-                            out_am = oam;
-                        }
                         if (own_diag) {
-                            if (!REG) Dg[i] = IO::ld(Mt + i * PM + i);
+                            Dg[i] = IO::ld(Mt + i * PM + i);
                             Mt[i * PM + i] = MS(0.f);
                         }
                     }
@@ -1134,9 +1109,6 @@ constexpr TierCfg kCfg32[kSmemTiers + 1] = {{0, 0, 0},     {32, 32, 1},  {64, 32
                                             {112, 28, 4}, {128, 32, 4}, {144, 36, 4}, {160, 40, 4}};
 constexpr TierCfg kCfg64[kSmemTiers + 1] = {{0, 0, 0},     {32, 16, 2},  {64, 16, 4},  {112, 28, 4},
                                             {112, 28, 4}, {112, 28, 4}, {112, 28, 4}, {112, 28, 4}};
-// FP32 tiers that keep their own outputs in registers (the others have no register room).
-constexpr bool kReg32[kSmemTiers + 1] = {false, true, true, false, false, true, false, false};
-
 // Bytes of one RW scratch slot: W [SMAX][SMAX] doubles, Dijkstra distances [warps][nodes]
 // doubles, parity [SMAX][SMAX] bytes, done and parity flags [warps][nodes] bytes.
 inline int64_t rw_slot_layout(int smax, int nt, int nodes) {
@@ -1151,10 +1123,10 @@ size_t smem_bytes_of() {
     return nref_offset<T, MS>(SMAX, G) + (sizeof(MS) == 2 ? (size_t)SMAX * sizeof(float) : 0) + (size_t)SMAX * 2 + 16;
 }
 
-template <typename T, int CH, int G, bool TRACE, bool REG, typename MS = T>
+template <typename T, int CH, int G, bool TRACE, typename MS = T>
 cudaError_t run_tier(const DecodeArgs& a, int num_sms, cudaStream_t st, bool prepare_only) {
     const size_t smem = smem_bytes_of<T, CH, G, MS>();
-    auto kern = decode_smem_kernel<T, CH, G, TRACE, REG, false, MS>;
+    auto kern = decode_smem_kernel<T, CH, G, TRACE, false, MS>;
     if (prepare_only)
         return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     int per_sm = 0;
@@ -1166,15 +1138,15 @@ cudaError_t run_tier(const DecodeArgs& a, int num_sms, cudaStream_t st, bool pre
 }
 
 // Every tier has a production instantiation and a traced one (tests).
-template <typename T, int CH, int G, bool REG, typename MS = T>
+template <typename T, int CH, int G, typename MS = T>
 cudaError_t run_tier2(const DecodeArgs& a, int num_sms, cudaStream_t st, bool prep) {
     const bool tr = a.tr_lambda != nullptr || a.tr_partner != nullptr;
     if (prep) {
-        cudaError_t e = run_tier<T, CH, G, false, REG, MS>(a, num_sms, st, true);
-        return e != cudaSuccess ? e : run_tier<T, CH, G, true, REG, MS>(a, num_sms, st, true);
+        cudaError_t e = run_tier<T, CH, G, false, MS>(a, num_sms, st, true);
+        return e != cudaSuccess ? e : run_tier<T, CH, G, true, MS>(a, num_sms, st, true);
     }
-    return tr ? run_tier<T, CH, G, true, REG, MS>(a, num_sms, st, false)
-              : run_tier<T, CH, G, false, REG, MS>(a, num_sms, st, false);
+    return tr ? run_tier<T, CH, G, true, MS>(a, num_sms, st, false)
+              : run_tier<T, CH, G, false, MS>(a, num_sms, st, false);
 }
 
 }  // namespace

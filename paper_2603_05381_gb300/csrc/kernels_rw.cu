@@ -12,11 +12,11 @@
 namespace bp4m {
 namespace {
 
-template <typename T, int CH, int G, bool REG>
+template <typename T, int CH, int G>
 cudaError_t rw_grid(int n_det, int num_sms, int* grid, int64_t* slot_bytes, size_t* smem_out) {
     constexpr int SMAX = CH * G, NT = CH * G * G;
     const size_t smem = smem_bytes_of<T, CH, G>();
-    auto kern = decode_smem_kernel<T, CH, G, false, REG, true>;
+    auto kern = decode_smem_kernel<T, CH, G, false, true>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     int per_sm = 0;
@@ -29,12 +29,12 @@ cudaError_t rw_grid(int n_det, int num_sms, int* grid, int64_t* slot_bytes, size
     return cudaSuccess;
 }
 
-template <typename T, int CH, int G, bool REG>
+template <typename T, int CH, int G>
 cudaError_t run_tier_rw(const DecodeArgs& a, int num_sms, cudaStream_t st, int64_t* query) {
     int grid = 0;
     int64_t slot = 0;
     size_t smem = 0;
-    cudaError_t e = rw_grid<T, CH, G, REG>(a.tb.n_det, num_sms, &grid, &slot, &smem);
+    cudaError_t e = rw_grid<T, CH, G>(a.tb.n_det, num_sms, &grid, &slot, &smem);
     if (e != cudaSuccess) return e;
     if (query) {
         query[0] = (int64_t)grid * slot;
@@ -44,7 +44,7 @@ cudaError_t run_tier_rw(const DecodeArgs& a, int num_sms, cudaStream_t st, int64
     // every block indexes its own slot: the scratch must hold grid slots of this tier's size
     if (a.gscratch == nullptr || a.rw_slot_bytes != slot || (int64_t)grid * slot > a.gscratch_bytes)
         return cudaErrorInvalidValue;
-    decode_smem_kernel<T, CH, G, false, REG, true><<<grid, CH * G * G, smem, st>>>(a);
+    decode_smem_kernel<T, CH, G, false, true><<<grid, CH * G * G, smem, st>>>(a);
     return cudaGetLastError();
 }
 
@@ -52,20 +52,20 @@ cudaError_t dispatch_rw(int precision, int tier, const DecodeArgs& a, int num_sm
                         int64_t* query) {
     if (precision == 0) {
         switch (tier) {
-            case 1: return run_tier_rw<double, 16, 2, false>(a, num_sms, st, query);
-            case 2: return run_tier_rw<double, 16, 4, false>(a, num_sms, st, query);
-            case 3: return run_tier_rw<double, 28, 4, false>(a, num_sms, st, query);
+            case 1: return run_tier_rw<double, 16, 2>(a, num_sms, st, query);
+            case 2: return run_tier_rw<double, 16, 4>(a, num_sms, st, query);
+            case 3: return run_tier_rw<double, 28, 4>(a, num_sms, st, query);
             default: return cudaErrorInvalidValue;
         }
     }
     switch (tier) {
-        case 1: return run_tier_rw<float, 32, 1, kReg32[1]>(a, num_sms, st, query);
-        case 2: return run_tier_rw<float, 32, 2, kReg32[2]>(a, num_sms, st, query);
-        case 3: return run_tier_rw<float, 24, 4, kReg32[3]>(a, num_sms, st, query);
-        case 4: return run_tier_rw<float, 28, 4, kReg32[4]>(a, num_sms, st, query);
-        case 5: return run_tier_rw<float, 32, 4, kReg32[5]>(a, num_sms, st, query);
-        case 6: return run_tier_rw<float, 36, 4, kReg32[6]>(a, num_sms, st, query);
-        case 7: return run_tier_rw<float, 40, 4, kReg32[7]>(a, num_sms, st, query);
+        case 1: return run_tier_rw<float, 32, 1>(a, num_sms, st, query);
+        case 2: return run_tier_rw<float, 32, 2>(a, num_sms, st, query);
+        case 3: return run_tier_rw<float, 24, 4>(a, num_sms, st, query);
+        case 4: return run_tier_rw<float, 28, 4>(a, num_sms, st, query);
+        case 5: return run_tier_rw<float, 32, 4>(a, num_sms, st, query);
+        case 6: return run_tier_rw<float, 36, 4>(a, num_sms, st, query);
+        case 7: return run_tier_rw<float, 40, 4>(a, num_sms, st, query);
         default: return cudaErrorInvalidValue;
     }
 }
