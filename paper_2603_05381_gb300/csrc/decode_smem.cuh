@@ -130,6 +130,20 @@ struct B2<double> {
     static __device__ __forceinline__ double mn(double a, double b) { return fmin(a, b); }
 };
 
+// Asynchronous global->shared copies: 16 bytes past L1, or 4 bytes
+__device__ __forceinline__ void cp_async16(void* smem_dst, const void* gmem_src) {
+    const unsigned d = (unsigned)__cvta_generic_to_shared(smem_dst);
+    const size_t g = __cvta_generic_to_global(gmem_src);
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(g) : "memory");
+}
+__device__ __forceinline__ void cp_async4(void* smem_dst, const void* gmem_src) {
+    const unsigned d = (unsigned)__cvta_generic_to_shared(smem_dst);
+    const size_t g = __cvta_generic_to_global(gmem_src);
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(d), "l"(g) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
 constexpr double kLog2e = 1.4426950408889634074;
 constexpr double kLn2 = 0.69314718055994530942;
 
@@ -222,11 +236,12 @@ __host__ __device__ constexpr int msg_pitch_of(int smax, int g) {
 
 // Byte offset of the 16-bit path's reference array in the dynamic shared memory, after
 // Mt, Lm, Dg, rowacc, dets, choice, bestp and matched (8-byte aligned).
+// With a helper warp there are two detector lists.
 template <typename T, typename MS>
-__host__ __device__ constexpr size_t nref_offset(int smax, int g) {
+__host__ __device__ constexpr size_t nref_offset(int smax, int g, bool help) {
     return (((size_t)smax * msg_pitch_of<T, MS>(smax, g) * sizeof(MS) + 15) / 16 * 16 +
             (size_t)(smax * pitch_of<T>(smax, g) + smax + (smax & 1)) * sizeof(T) +
-            (size_t)smax * (sizeof(double) + 2 * sizeof(int) + sizeof(short) + 1) + 7) / 8 * 8;
+            (size_t)smax * (sizeof(double) + (help ? 3 : 2) * sizeof(int) + sizeof(short) + 1) + 7) / 8 * 8;
 }
 
 // A thread's register-cached row entries (CH columns).  FP32 keeps them as float2 pairs,
@@ -287,31 +302,52 @@ __device__ __forceinline__ void combine_max(T& m1, T& m2, int& k, T o1, T o2, in
     }
 }
 
-// Blocks per SM the kernel is compiled for: the FP32 384- and 448-thread tiers (96 and 112
-// rows, 79 and 106 KB of shared memory) run two blocks per SM, and so does the 512-thread
-// tier (128 rows) with 16-bit messages (102 KB); the others are limited by shared memory or
-// 128 registers.
+// Blocks per SM the kernel is compiled for.  FP32 arithmetic: as many as shared memory holds
+// and registers allow without spills: nine of 96 threads (48 rows), six of 128 (64 rows), three of
+// 320 (80 rows), two of 384 and 448 (96 and 112 rows; 79 and 106 KB), and two of 512 (128 rows)
+// with 16-bit messages (102 KB); the others are limited by shared memory or 128 registers.
 __host__ __device__ constexpr int blocks_for(int nt, int elem_bytes, int msg_bytes) {
-    return (elem_bytes == 4 && (nt == 384 || nt == 448 || (nt == 512 && msg_bytes == 2))) ? 2 : min_blocks(nt);
+    if (elem_bytes != 4) return min_blocks(nt);
+    return nt == 96 ? 9 : nt == 128 ? 6 : nt == 320 ? 3 : nt == 384 || nt == 448 ? 2 : nt == 512 && msg_bytes == 2 ? 2 : min_blocks(nt);
 }
 
-// Rows watched for the convergence decision (FP32 arithmetic): a shot has converged only if
-// every row keeps exactly one variable, so one row that does not settles an iteration's
-// decision.  kWatch warps each look at one row that was seen violating; only when all of them
-// have stopped violating is every row counted.  Counting every row in every iteration took an
-// add, a multiply and an own-output read per message, or a register copy of the outputs (24
-// warp instructions per 32 updates at 144 rows, 19 without); measured on 200,001 d = 21
-// code-capacity shots 99.9 -> 88.2 ms, 300,000 d = 13 circuit shots 281.4 -> 269.0 ms, 10^6
-// d = 9 code-capacity shots 16.0 -> 14.3 ms, outputs equal.
+// Convergence decision (FP32 arithmetic).  A shot has converged only if every row keeps exactly
+// one variable, so one row that does not settles an iteration's decision.  The block's last warp
+// watches kWatch rows that were seen violating; only when none of them violates is every row
+// counted (in about 1% of the iterations of d = 13 circuit shots, 20 of whose rows violate in the
+// median iteration).  Counting every row in every iteration took an add, a multiply and an
+// own-output read per message, or a register copy of the outputs (24 warp instructions per 32
+// updates at 144 rows, 19 without).
+//
+// Bound: the special-function unit takes 0.094 SM-cycles an update (ex2 and lg2), the compares
+// and maxima of the row scan about as much; the phases of an iteration run one after another
+// between its two barriers, so that the tiers of one block per SM reach about 0.3 of that.
+// Measured per tier (d = 13 circuit, 100,000 shots; G updates/s at the start and now): 96 rows
+// 888 -> 1035, 112 rows 1004 -> 1189, 128 rows 875 -> 994, 144 rows 836 -> 970, 160 rows
+// 906 -> 1054; 64 rows (d = 21 code capacity) 1039 -> 1325.  Double-buffered messages with the
+// priors in registers (one barrier an iteration, half the shared-memory reads) measured the same
+// or slower: 96 registers a thread made it spill.
 constexpr int kWatch = 4;
+
+// The FP32-arithmetic forms of 128 and 144 rows that run one block per SM have a helper warp: it
+// watches beside the others' reads instead of holding up the vote, and fetches the next shot's
+// detector list during the first iteration.  (160 rows: twenty warps of 96 registers leave no
+// room for it.  Where two blocks share an SM the other block fills the gaps.)
+__host__ __device__ constexpr bool helper_warp(int smax, int elem_bytes, int msg_bytes, bool rw) {
+    return elem_bytes == 4 && !rw && (smax == 144 || (smax == 128 && msg_bytes == 4));
+}
+__host__ __device__ constexpr int block_threads(int ch, int g, int elem_bytes, int msg_bytes, bool rw) {
+    return ch * g * g + (helper_warp(ch * g, elem_bytes, msg_bytes, rw) ? 32 : 0);
+}
 
 // RW = true: the B-BP4MF second stage.  The shot's priors, pair weights and parities are
 // computed in the block by Dijkstra from every defect over per-qubit weights derived from
 // the first stage's posteriors (instead of being gathered from the static tables).
 template <typename T, int CH, int G, bool TRACE, bool RW = false, typename MS = T>
-__global__ void __launch_bounds__(CH * G * G, blocks_for(CH * G * G, (int)sizeof(T), (int)sizeof(MS))) decode_smem_kernel(const DecodeArgs a) {
+__global__ void __launch_bounds__(block_threads(CH, G, (int)sizeof(T), (int)sizeof(MS), RW), blocks_for(CH * G * G, (int)sizeof(T), (int)sizeof(MS))) decode_smem_kernel(const DecodeArgs a) {
     constexpr int SMAX = CH * G;
-    constexpr int NT = SMAX * G;
+    constexpr bool HELP = helper_warp(SMAX, (int)sizeof(T), (int)sizeof(MS), RW);
+    constexpr int NT = block_threads(CH, G, (int)sizeof(T), (int)sizeof(MS), RW);
     constexpr int R = 32 / G;
     constexpr int P = pitch_of<T>(SMAX, G);          // priors
     constexpr int PM = msg_pitch_of<T, MS>(SMAX, G);  // messages
@@ -321,18 +357,19 @@ __global__ void __launch_bounds__(CH * G * G, blocks_for(CH * G * G, (int)sizeof
     static_assert(NT % 32 == 0 && NT <= 1024, "block size");
     using Mask = typename std::conditional<(CH > 32), unsigned long long, unsigned int>::type;
     extern __shared__ __align__(16) unsigned char smem[];
-    MS* Mt = reinterpret_cast<MS*>(smem);        // Mt[i][k] = M[k][i]; diagonal kept 0
-    T* Lm = reinterpret_cast<T*>(smem + ((size_t)SMAX * PM * sizeof(MS) + 15) / 16 * 16);  // Lm[i][k] = l_ik (log2), -inf past s
-    T* Dg = Lm + SMAX * P;                          // Dg[i] = M[i][i] (factor i to its boundary variable)
+    MS* const Mt = reinterpret_cast<MS*>(smem);  // Mt[i][k] = M[k][i]; diagonal kept 0
+    T* const Lm = reinterpret_cast<T*>(smem + ((size_t)SMAX * PM * sizeof(MS) + 15) / 16 * 16);  // Lm[i][k] = l_ik (log2), -inf past s
+    T* const Dg = Lm + SMAX * P;                 // Dg[i] = M[i][i] (factor i to its boundary variable)
     double* rowacc = reinterpret_cast<double*>(Dg + SMAX + (SMAX & 1));
-    int* dets = reinterpret_cast<int*>(rowacc + SMAX);
-    int* choice = dets + SMAX;
+    int* const dets0 = reinterpret_cast<int*>(rowacc + SMAX);
+    int* dets = dets0;  // HELP: the current one of two
+    int* choice = dets0 + (HELP ? 2 : 1) * SMAX;
     short* bestp = reinterpret_cast<short*>(choice + SMAX);
     unsigned char* matched = reinterpret_cast<unsigned char*>(bestp + SMAX);
     // 16-bit messages: nrefv[k] = -r_k, minus the reference of the messages leaving factor k
-    float* nrefv = reinterpret_cast<float*>(smem + nref_offset<T, MS>(SMAX, G));
+    float* const nrefv = reinterpret_cast<float*>(smem + nref_offset<T, MS>(SMAX, G, HELP));
     // static-partition forced convergence: factors in processing order
-    short* order = reinterpret_cast<short*>(smem + nref_offset<T, MS>(SMAX, G) + (HALF ? (size_t)SMAX * 4 : 0));
+    short* order = reinterpret_cast<short*>(smem + nref_offset<T, MS>(SMAX, G, HELP) + (HALF ? (size_t)SMAX * 4 : 0));
     // RW only: per-shot W (FP64) and parity over local ranks, Dijkstra state per warp, in
     // this block's global scratch slot (layout of rw_slot_layout)
     const int rw_nodes = a.tb.n_det + 1;
@@ -343,8 +380,11 @@ __global__ void __launch_bounds__(CH * G * G, blocks_for(CH * G * G, (int)sizeof
     unsigned char* Psh = reinterpret_cast<unsigned char*>(rw_dist + (NT / 32) * rw_nodes);
     unsigned char* rw_done = Psh + SMAX * SMAX;
     unsigned char* rw_par = rw_done + (NT / 32) * rw_nodes;
-    __shared__ int sh_item, sh_s, sh_best_par, sh_best_forced, sh_improve, sh_use_best;
+    __shared__ int sh_item, sh_s, sh_flags, sh_best_par, sh_best_forced, sh_improve, sh_use_best;
     __shared__ double sh_best_w;
+    __shared__ int sh_next_code[2], sh_next_s[2];  // HELP: the shots fetched ahead
+    __shared__ unsigned sh_open[(SMAX + 31) / 32];  // forced convergence: unmatched rows
+    __shared__ int sh_watch[kWatch];
     __shared__ unsigned sh_bad[NT / 32];  // full count: each warp's rows that do not keep exactly one
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -371,12 +411,14 @@ __global__ void __launch_bounds__(CH * G * G, blocks_for(CH * G * G, (int)sizeof
     MS* const row_m = Mt + i * PM + k0;  // incoming messages M[k][i]
     MS* const col_m = Mt + k0 * PM + i;  // own outputs M[i][k] live at Mt[k][i], register c at [col_off(c) PM]
 #define COL(c) (k0 + col_off<PAIR, G>(c))
-#define RL(c) row_l[col_off<PAIR, G>(c)]
+#define RL(c) l_ld1(c)
 #define RM(c) m_ld1(row_m + col_off<PAIR, G>(c), COL(c))
 #define CMP(c) (col_m + col_off<PAIR, G>(c) * PM)
 #define CM(c) m_ld1(CMP(c), i)
-#define RL2(j) (*reinterpret_cast<const float2*>(row_l + col_off<PAIR, G>(2 * (j))))
+#define RL2(j) l_ld2(j)
 #define RM2(j) m_ld2(row_m + col_off<PAIR, G>(2 * (j)), k0 + col_off<PAIR, G>(2 * (j)))
+    auto l_ld1 = [&](int c) -> T { return row_l[col_off<PAIR, G>(c)]; };
+    auto l_ld2 = [&](int j) -> float2 { return *reinterpret_cast<const float2*>(row_l + col_off<PAIR, G>(2 * j)); };
     // messages arriving at row i from columns k, k + 1 (16-bit: decoded with the source rows'
     // references), and one arriving from column k
     auto m_ld2 = [&](const MS* p, int k) -> float2 {
@@ -392,36 +434,74 @@ __global__ void __launch_bounds__(CH * G * G, blocks_for(CH * G * G, (int)sizeof
             return IO::ld(p);
     };
 
-    for (;;) {
-        if (tid == 0) sh_item = atomicAdd(a.next, 1);
-        __syncthreads();
-        const int item = sh_item;
-        if (item >= count) break;
-        const ItemCtx ic = resolve_item(a, a.list[item]);
-        const int64_t shot = ic.shot;
-        const int n = ic.tb.n_det;
-        const T* __restrict__ Ltab = Num<T>::L(ic.tb);
-        if (warp == 0) {
-            const int s0 = compact_defects(ic.synd + (size_t)shot * ic.tb.n_words, ic.tb.n_words,
-                                           dets, SMAX, lane);
-            if (lane == 0) sh_s = s0;
+    // HELP: the last warp takes the block's next item into buffer b (code -1: none left)
+    auto fetch_next = [&](int b) {
+        int item = 0;
+        if (lane == 0) item = atomicAdd(a.next, 1);
+        item = __shfl_sync(kFull, item, 0);
+        int c = -1, s0 = 0;
+        if (item < count) {
+            c = a.list[item];
+            const ItemCtx ic = resolve_item(a, c);
+            s0 = compact_defects(ic.synd + (size_t)ic.shot * ic.tb.n_words, ic.tb.n_words, dets0 + b * SMAX, SMAX, lane);
         }
+        if (lane == 0) {
+            sh_next_code[b] = c;
+            sh_next_s[b] = s0;
+        }
+    };
+    int pb = 0;
+    if (HELP) {
+        if (warp == NT / 32 - 1) fetch_next(0);
         __syncthreads();
-        const int s = sh_s;
-        if (s > SMAX || s < 1) {
+    }
+
+    for (;;) {
+        // the graph and outputs are looked up where they are needed: kept across the iterations
+        // they would take twenty registers
+        int code, s;
+        if constexpr (HELP) {
+            code = sh_next_code[pb];
+            if (code < 0) break;
+            s = sh_next_s[pb];
+            dets = dets0 + pb * SMAX;
+        } else {
+            if (tid == 0) sh_item = atomicAdd(a.next, 1);
+            __syncthreads();
+            const int item = sh_item;
+            if (item >= count) break;
+            code = a.list[item];
+            if (warp == 0) {
+                const ItemCtx ic = resolve_item(a, code);
+                const int s0 = compact_defects(ic.synd + (size_t)ic.shot * ic.tb.n_words, ic.tb.n_words, dets, SMAX, lane);
+                if (lane == 0) sh_s = s0;
+            }
+            __syncthreads();
+            s = sh_s;
+        }
+        const ItemCtx ic0 = resolve_item(a, code);
+        const int64_t shot = ic0.shot;
+        const int n = ic0.tb.n_det;
+        const T* __restrict__ Ltab = Num<T>::L(ic0.tb);
+        if (s > SMAX || s < (HELP ? 2 : 1)) {
             if (tid == 0 && a.ctr) atomicAdd(a.ctr + C_ERRORS, 1ull);
+            if constexpr (HELP) {
+                __syncthreads();
+                if (warp == NT / 32 - 1) fetch_next(pb);
+                __syncthreads();
+            }
             continue;
         }
         const bool tr_on = TRACE && s <= a.s_cap;
-        if (s == 1 && !RW) {
+        if (!HELP && s == 1 && !RW) {
             // a single factor with a single variable: the leave-one-out set is empty, the
             // message is +inf and v_00 is kept in every iteration
             if (tid == 0) {
                 const int its = full ? a.T : 1;
                 const int d0 = dets[0];
-                if (ic.obs_pred) ic.obs_pred[shot] = ic.tb.P[(size_t)d0 * n + d0];
-                if (ic.flags) ic.flags[shot] = F_CONVERGED;
-                if (ic.iters) ic.iters[shot] = (int16_t)its;
+                if (ic0.obs_pred) ic0.obs_pred[shot] = ic0.tb.P[(size_t)d0 * n + d0];
+                if (ic0.flags) ic0.flags[shot] = F_CONVERGED;
+                if (ic0.iters) ic0.iters[shot] = (int16_t)its;
                 if (tr_on && trl) trl[(size_t)shot * a.s_cap * a.s_cap] = Num<T>::pinf();
                 if (tr_on && a.tr_partner) {
                     a.tr_partner[(size_t)shot * a.s_cap] = 0;
@@ -434,9 +514,39 @@ __global__ void __launch_bounds__(CH * G * G, blocks_for(CH * G * G, (int)sizeof
             }
             continue;
         }
+        const bool act = i < s;
+        // rows warp*R .. warp*R+R-1 belong to this warp; a warp with none of them active
+        // skips the read and compute phases (it still takes part in every barrier)
+        const bool wact = warp * R < s;
+        Regs<T, CH> q;
         // ---- gather the shot's priors (log2 units); columns past s are -inf so that they
         // never win a max, add nothing to a sum and are never kept
-        if (!RW) {
+        if constexpr (std::is_same<T, float>::value && !RW) {
+            // The table is symmetric: each pair k >= r is fetched once, row by row (a warp's 32
+            // columns of one table row lie in about ten 128-byte lines), with every copy of the
+            // shot in flight at once, and mirrored in shared memory.
+            float* const st = reinterpret_cast<float*>(Lm);
+            for (int r = warp; r < s; r += NT / 32) {
+                const T* trow = Ltab + (size_t)dets[r] * n;
+                for (int k = r + lane; k < s; k += 32) cp_async4(st + r * P + k, trow + dets[k]);
+            }
+            cp_async_commit();
+            cp_async_wait_all();
+            __syncthreads();
+#pragma unroll
+            for (int c = 0; c < CH; ++c) {
+                const int k = COL(c);
+                q[c] = act && k < s ? st[k >= i ? i * P + k : k * P + i] * (float)kLog2e : ninf;
+            }
+            __syncthreads();
+            if (act) {
+#pragma unroll
+                for (int c = 0; c < CH; ++c) {
+                    row_l[col_off<PAIR, G>(c)] = q[c];
+                    row_m[col_off<PAIR, G>(c)] = MS(0.f);
+                }
+            }
+        } else if (!RW) {
             for (int r = warp; r < s; r += NT / 32) {
                 const T* trow = Ltab + (size_t)dets[r] * n;
                 for (int k = lane; k < SMAX; k += 32) {
@@ -534,6 +644,7 @@ __global__ void __launch_bounds__(CH * G * G, blocks_for(CH * G * G, (int)sizeof
             if constexpr (HALF) nrefv[tid] = 0.f;
         }
         if (tid == 0) {
+            sh_flags = 0;
             sh_best_w = Num<double>::pinf();
             sh_best_par = 0;
             sh_best_forced = 0;
@@ -544,9 +655,9 @@ __global__ void __launch_bounds__(CH * G * G, blocks_for(CH * G * G, (int)sizeof
             // one defect: matched to the boundary along its reweighted path
             if (tid == 0) {
                 const int its = full ? a.T : 1;
-                if (ic.obs_pred) ic.obs_pred[shot] = Psh[0];
-                if (ic.flags) ic.flags[shot] = F_CONVERGED;
-                if (ic.iters) ic.iters[shot] = (int16_t)its;
+                if (ic0.obs_pred) ic0.obs_pred[shot] = Psh[0];
+                if (ic0.flags) ic0.flags[shot] = F_CONVERGED;
+                if (ic0.iters) ic0.iters[shot] = (int16_t)its;
                 acc_it += (unsigned long long)its;
                 acc_msg += (unsigned long long)its;
                 acc_def += 1;
@@ -555,53 +666,163 @@ __global__ void __launch_bounds__(CH * G * G, blocks_for(CH * G * G, (int)sizeof
             continue;
         }
 
-        const bool act = i < s;
-        // rows warp*R .. warp*R+R-1 belong to this warp; a warp with none of them active
-        // skips the read and compute phases (it still takes part in every barrier)
-        const bool wact = warp * R < s;
-        Regs<T, CH> q;
-        constexpr int NWATCH = NT / 32 < kWatch ? NT / 32 : kWatch;
-        int watch = warp < NWATCH ? warp * s / NWATCH : 0;  // this warp's watched row
+        constexpr int WW = NT / 32 - 1;  // the warp that watches
+        int wj = 0;                      // the watched row tried first
         int t = 0;
-        bool any_conv = false, forced_ran = false;
-        int out_par = 0, out_forced = 0, out_from_best = 0;
-        int partner = -1;
+        // set where a candidate finishes the shot
+        int out_par, out_forced, out_from_best, partner;
 
-        for (;;) {
-            // ---- read phase: Q = l + M[k][i]/alpha for the next update.  FP32: the row's maximum /
-            // second maximum scan of the next update runs in the same loop (it needs only Q), so
-            // that the shared-memory loads and the scan's ALU work overlap.  The marginalization of
-            // lambda^t = l + (M[i][k] + M[k][i]) (t > 0) is not evaluated here: see the watched rows
-            // below.
-            Mask bits = 0;
-            float sa1 = Num<float>::ninf(), sa2 = Num<float>::ninf();
-            int sab = 0;
-            // (max, second max, first block of the max) over the blocks of four columns so far.
-            // Only the block of four is tracked (one compare and one select for four columns
-            // instead of two per column: the compare, select and max instructions bound this
-            // phase); the thread that holds the row's maximum finds the column in its block
-            // afterwards.
-            auto scan4 = [&](int b, float2 p0, float2 p1) {
-                const float h0 = fmaxf(p0.x, p0.y), l0 = fminf(p0.x, p0.y);
-                const float h1 = fmaxf(p1.x, p1.y), l1 = fminf(p1.x, p1.y);
-                const float hi = fmaxf(h0, h1), lo = max3f(l0, l1, fminf(h0, h1));
-                sab = hi > sa1 ? b : sab;
-                sa2 = max3f(sa2, lo, fminf(sa1, hi));
-                sa1 = fmaxf(sa1, hi);
-            };
-            if (!wact) {
-            } else if (!act) {
+        // FP32: Q = l + M[k][i]/alpha for the next update, with the row's maximum m1 and second
+        // maximum m2 scanned in the same loop (it needs only Q), so that the shared-memory loads
+        // and the scan's ALU work overlap.  The column of m1 is not tracked here: the exponential
+        // loop below finds it as the one column above m2.
+        T m1 = ninf, m2 = ninf;
+        auto read_rows = [&]() {
+          if constexpr (std::is_same<T, float>::value) {
+            if (!wact) return;
+            m1 = ninf;
+            m2 = ninf;
+            if (!act) {
 #pragma unroll
                 for (int c = 0; c < CH; ++c) q[c] = ninf;
-            } else if constexpr (std::is_same<T, float>::value) {
+            } else {
                 const float2 ainv2 = make_float2(ainv, ainv);
 #pragma unroll
                 for (int j = 0; j < CH / 2; j += 2) {
-                    q.p[j] = __ffma2_rn(RM2(j), ainv2, RL2(j));
-                    q.p[j + 1] = __ffma2_rn(RM2(j + 1), ainv2, RL2(j + 1));
-                    scan4(j / 2, q.p[j], q.p[j + 1]);
+                    const float2 p0 = __ffma2_rn(RM2(j), ainv2, RL2(j));
+                    const float2 p1 = __ffma2_rn(RM2(j + 1), ainv2, RL2(j + 1));
+                    q.p[j] = p0;
+                    q.p[j + 1] = p1;
+                    // four columns' maximum and second maximum into the row's
+                    const float h0 = fmaxf(p0.x, p0.y), l0 = fminf(p0.x, p0.y);
+                    const float h1 = fmaxf(p1.x, p1.y), l1 = fminf(p1.x, p1.y);
+                    const float hi = fmaxf(h0, h1), lo = max3f(l0, l1, fminf(h0, h1));
+                    m2 = max3f(m2, lo, fminf(m1, hi));
+                    m1 = fmaxf(m1, hi);
                 }
-                if (TRACE && tr_on && trl && t > 0) {
+            }
+#pragma unroll
+            for (int off = R; off < 32; off <<= 1) {
+                const T o1 = __shfl_xor_sync(kFull, m1, off);
+                const T o2 = __shfl_xor_sync(kFull, m2, off);
+                m2 = max3f(m2, o2, fminf(m1, o1));
+                m1 = fmaxf(m1, o1);
+            }
+          }
+        };
+        // FP32: leave-one-out max* of every row.  With m1 (at column am) and m2 the two largest Q of
+        // the row and S = sum_k min(2^(Q_k - m2), 1), so that S - 1 = sum_{k != am} 2^(Q_k - m2) >= 1:
+        //   k != am: M'[i][k] = -(m1 + lg2(1 + 2^(m2 - m1) (S - 1 - 2^(Q_k - m2))))
+        //   k == am: M'[i][k] = -(m2 + lg2(S - 1))
+        // (the generic value is written for every column, the thread with a column above m2 then
+        // overwrites it; where m1 == m2 no column is above m2 and both formulas give the same
+        // value: 2^(m2 - m1) = 1 and S - 1 is exact).  Row i's outputs M'[i][k] go to Mn[k][i].
+        auto update_rows = [&]() {
+          if constexpr (std::is_same<T, float>::value) {
+            if (!wact) return;
+            // 2^(Q - m2) from m2 - Q, whose sign bit marks the column above m2: one funnel shift a
+            // column collects them, first column in the highest bit
+            const float2 m22 = make_float2(m2, m2), neg1 = make_float2(-1.f, -1.f);
+            float2 s2 = make_float2(0.f, 0.f);
+            unsigned top0 = 0, top1 = 0;
+#pragma unroll
+            for (int j = 0; j < CH / 2; ++j) {
+                const float2 dq = __ffma2_rn(q.p[j], neg1, m22);
+                const float2 u = make_float2(B2<float>::ex2(-dq.x), B2<float>::ex2(-dq.y));
+                q.p[j] = u;
+                s2 = __fadd2_rn(s2, make_float2(sat1(u.x), sat1(u.y)));
+                unsigned& top = j < 16 ? top0 : top1;
+                top = __funnelshift_l(__float_as_uint(dq.x), top, 1);
+                top = __funnelshift_l(__float_as_uint(dq.y), top, 1);
+            }
+            float S32 = s2.x + s2.y;
+#pragma unroll
+            for (int off = R; off < 32; off <<= 1) S32 += __shfl_xor_sync(kFull, S32, off);
+            if (!act) return;
+            const float cf32 = B2<float>::ex2(m2 - m1);
+            const float Aa32 = __fmaf_rn(cf32, S32 - 1.f, 1.f);
+            // 16-bit storage: this row's reference r_i = m1 rounded to the format (so that it is
+            // exact there); stored values out + r_i = -lg2(Aa - cf u) + (r_i - m1)
+            float rf = 0.f, dref32 = 0.f;
+            if constexpr (HALF) {
+                rf = IO::unpack(IO::pack(m1, 0.f)).x;
+                dref32 = rf - m1;
+            }
+            // out = -m1 - lg2(Aa - cf u), the subtraction as an exact fma with -1
+            const float2 ncf = make_float2(-cf32, -cf32), A2 = make_float2(Aa32, Aa32);
+            const float2 nm1 = HALF ? make_float2(dref32, dref32) : make_float2(-m1, -m1);
+#pragma unroll
+            for (int j = 0; j < CH / 2; ++j) {
+                const float2 y = __ffma2_rn(ncf, q.p[j], A2);
+                const float2 lg = make_float2(B2<float>::lg2(y.x), B2<float>::lg2(y.y));
+                const float2 out = __ffma2_rn(lg, neg1, nm1);
+                if constexpr (HALF) {
+                    // store the rounded pair (relative to r_i): both ends of a variable read the
+                    // same message
+                    const unsigned pk2 = IO::pack(out.x, out.y);
+                    *reinterpret_cast<unsigned short*>(CMP(2 * j)) = (unsigned short)(pk2 & 0xFFFFu);
+                    *reinterpret_cast<unsigned short*>(CMP(2 * j + 1)) = (unsigned short)(pk2 >> 16);
+                } else {
+                    *CMP(2 * j) = out.x;
+                    *CMP(2 * j + 1) = out.y;
+                }
+            }
+            if (top0 | top1) {
+                constexpr int N0 = CH < 32 ? CH : 32;
+                const int c = top0 ? N0 - 32 + __clz((int)top0) : CH - 32 + __clz((int)top1);
+                const int am = COL(c);
+                const float lgS = B2<float>::lg2(S32 - 1.f);
+                if constexpr (HALF)
+                    IO::st(Mt + am * PM + i, __fmaf_rn(lgS, -1.f, rf - m2));
+                else
+                    IO::st(Mt + am * PM + i, -m2 - lgS);
+            }
+            if (own_diag) {
+                MS* const md = Mt + i * PM + i;
+                if constexpr (HALF) {
+                    // the diagonal holds r_i, which decodes to exactly 0
+                    Dg[i] = IO::ld(md) + (-rf);
+                    IO::st(md, rf);
+                    nrefv[i] = -rf;
+                } else {
+                    Dg[i] = IO::ld(md);
+                    *md = MS(0.f);
+                }
+            }
+          }
+        };
+        if (tid < kWatch) sh_watch[tid] = tid * s / kWatch;
+        // FP32: 1 if a watched row does not keep exactly one variable of lambda^t.  The rows are tried
+        // from the one that violated last; one that keeps exactly one moves on.
+        auto watch_rows = [&]() -> int {
+          if constexpr (std::is_same<T, float>::value) {
+            for (int tries = 0; tries < kWatch; ++tries) {
+                const int r = sh_watch[wj];
+                int cnt = 0;
+#pragma unroll
+                for (int j = 0; j < (SMAX + 31) / 32; ++j) {
+                    const int k = min(lane + 32 * j, s - 1);
+                    const float l = Lm[r * P + k];
+                    const float lam = k == r ? l + Dg[r] : l + (m_ld1(Mt + k * PM + r, r) + m_ld1(Mt + r * PM + k, k));
+                    cnt += lane + 32 * j < s && lam > 0.f ? 1 : 0;
+                }
+                if (__reduce_add_sync(kFull, cnt) != 1) return 1;
+                if (lane == 0) sh_watch[wj] = r + 1 < s ? r + 1 : 0;
+                wj = (wj + 1) % kWatch;
+                __syncwarp();
+            }
+            return 0;
+          }
+          return 1;
+        };
+
+        for (;;) {
+            // ---- convergence of lambda^t: every row keeps exactly one variable; the watched row
+            // settles most votes (in a d = 13 circuit shot 20 rows violate in the median iteration)
+            Mask bits = 0;
+            int conv = 0, chosen = -1;
+            if constexpr (std::is_same<T, float>::value) {
+                if (TRACE && tr_on && trl && t > 0 && act) {
 #pragma unroll
                     for (int c = 0; c < CH; ++c) {
                         const int k = COL(c);
@@ -610,8 +831,55 @@ __global__ void __launch_bounds__(CH * G * G, blocks_for(CH * G * G, (int)sizeof
                                 (k == i ? RL(c) + Dg[i] : RL(c) + (CM(c) + RM(c))) * (float)kLn2;
                     }
                 }
+                read_rows();
+                {
+                    int violated = t == 0;
+                    if (warp == WW) {
+                        if (t > 0) violated = watch_rows();
+                        if (HELP && t == 0) fetch_next(pb ^ 1);
+                    }
+                    // (also the barrier between reading Mt and overwriting it)
+                    conv = !__syncthreads_or(violated);
+                    if (conv) {
+                        // no watched row violates: count every row, and find its kept column
+                        int k1 = -1, cnt = 0;
+                        if (act) {
+#pragma unroll
+                            for (int c = 0; c < CH; ++c) {
+                                const int k = COL(c);
+                                const float l = RL(c);
+                                const float lam = k == i ? l + Dg[i] : l + (CM(c) + RM(c));
+                                cnt += lam > 0.f ? 1 : 0;
+                                if (lam > 0.f) k1 = k;
+                            }
+                        }
+#pragma unroll
+                        for (int off = R; off < 32; off <<= 1) {
+                            cnt += __shfl_xor_sync(kFull, cnt, off);
+                            k1 = max(k1, __shfl_xor_sync(kFull, k1, off));
+                        }
+                        chosen = k1;
+                        const bool bad = act && cnt != 1;
+                        const unsigned badrows = __ballot_sync(kFull, bad) & (R == 32 ? kFull : (1u << (R & 31)) - 1u);
+                        if (lane == 0) sh_bad[warp] = badrows;
+                        conv = __syncthreads_and(!bad);
+                        if (!conv && warp == WW) {
+                            // watch violating rows, the first at or after each share of the rows
+                            for (int j = 0; j < kWatch; ++j) {
+                                int w = j * (NT / 32) / kWatch;
+                                while (sh_bad[w] == 0u) w = w + 1 < NT / 32 ? w + 1 : 0;
+                                if (lane == 0) sh_watch[j] = w * R + __ffs((int)sh_bad[w]) - 1;
+                            }
+                        }
+                    }
+                }
             } else {
-                if (t == 0) {
+                // FP64: every row is counted in the read phase
+                if (!wact) {
+                } else if (!act) {
+#pragma unroll
+                    for (int c = 0; c < CH; ++c) q[c] = ninf;
+                } else if (t == 0) {
 #pragma unroll
                     for (int c = 0; c < CH; ++c) q[c] = B2<T>::fma_(RM(c), ainv, RL(c));
                 } else {
@@ -637,90 +905,6 @@ __global__ void __launch_bounds__(CH * G * G, blocks_for(CH * G * G, (int)sizeof
                         if (tr_on && trl) trl[((size_t)shot * a.s_cap + i) * a.s_cap + i] = lam * (T)kLn2;
                     }
                 }
-            }
-            // FP32: the row's (m1, m2) of the next update over the G threads, and the column of m1
-            // in the thread that holds it (own_max).  No index travels with the maxima: where
-            // m1 > m2 exactly one thread holds m1, and where m1 == m2 the generic output formula and
-            // the one for the maximum's column give the same value (2^(m2 - m1) = 1, and S - 1 is
-            // exact), so any holder may write it.
-            T m1 = ninf, m2 = ninf;
-            int am = 0x7fffffff;
-            bool own_max = false;
-            int conv, chosen = -1;
-            if constexpr (std::is_same<T, float>::value) {
-                if (wact) {
-                    m1 = sa1;
-                    m2 = sa2;
-#pragma unroll
-                    for (int off = R; off < 32; off <<= 1) {
-                        const T o1 = __shfl_xor_sync(kFull, m1, off);
-                        const T o2 = __shfl_xor_sync(kFull, m2, off);
-                        m2 = max3f(m2, o2, fminf(m1, o1));
-                        m1 = fmaxf(m1, o1);
-                    }
-                    own_max = act && sa1 == m1;
-                    if (own_max) {
-                        // the same values as in the loop above: Mt is still as it was read
-                        const float2 ainv2 = make_float2(ainv, ainv);
-                        const float2 p0 = __ffma2_rn(m_ld2(row_m + 4 * G * sab, k0 + 4 * G * sab), ainv2,
-                                                     *reinterpret_cast<const float2*>(row_l + 4 * G * sab));
-                        const float p1x = __fmaf_rn(m_ld1(row_m + 4 * G * sab + 2 * G, k0 + 4 * G * sab + 2 * G), ainv,
-                                                    row_l[4 * G * sab + 2 * G]);
-                        am = k0 + 4 * G * sab + (p0.x == m1 ? 0 : p0.y == m1 ? 1 : p1x == m1 ? 2 * G : 2 * G + 1);
-                    }
-                }
-                // ---- convergence of lambda^t.  The watched rows are counted by one warp each; a
-                // single row that does not keep exactly one variable settles the vote (one reader
-                // warp per row costs a few tens of instructions, counting every row an add, a
-                // compare and two shared-memory reads per message).  In a d = 13 circuit shot 20
-                // rows violate in the median iteration, so the full count runs in about 1% of them
-                // besides the ones that converge.
-                int violated = t == 0;
-                if (t > 0 && warp < NWATCH) {
-                    const int r = watch;
-                    int cnt = 0;
-#pragma unroll
-                    for (int k = lane; k < SMAX; k += 32) {
-                        const float l = Lm[r * P + k];
-                        const float lam = k == r ? l + Dg[r] : l + (m_ld1(Mt + k * PM + r, r) + m_ld1(Mt + r * PM + k, k));
-                        cnt += lam > 0.f ? 1 : 0;
-                    }
-                    violated = __reduce_add_sync(kFull, cnt) != 1;
-                    if (!violated) watch = r + 1 < s ? r + 1 : 0;
-                }
-                // (also the barrier between reading Mt and overwriting it)
-                conv = !__syncthreads_or(violated);
-                if (conv) {
-                    // no watched row violates: count every row, and find its kept column
-                    int k1 = -1, cnt = 0;
-                    if (act) {
-#pragma unroll
-                        for (int c = 0; c < CH; ++c) {
-                            const int k = COL(c);
-                            const float l = RL(c);
-                            const float lam = k == i ? l + Dg[i] : l + (CM(c) + RM(c));
-                            cnt += lam > 0.f ? 1 : 0;
-                            if (lam > 0.f) k1 = k;
-                        }
-                    }
-#pragma unroll
-                    for (int off = R; off < 32; off <<= 1) {
-                        cnt += __shfl_xor_sync(kFull, cnt, off);
-                        k1 = max(k1, __shfl_xor_sync(kFull, k1, off));
-                    }
-                    chosen = k1;
-                    const bool bad = act && cnt != 1;
-                    const unsigned badrows = __ballot_sync(kFull, bad) & (R == 32 ? kFull : (1u << (R & 31)) - 1u);
-                    if (lane == 0) sh_bad[warp] = badrows;
-                    conv = __syncthreads_and(!bad);
-                    if (!conv && warp < NWATCH) {
-                        // watch the first violating row at or after this warp's share of the rows
-                        int w = warp * (NT / 32) / NWATCH;
-                        while (sh_bad[w] == 0u) w = w + 1 < NT / 32 ? w + 1 : 0;
-                        watch = w * R + __ffs((int)sh_bad[w]) - 1;
-                    }
-                }
-            } else {
                 // kept count << 16 plus (first kept column + 1), summed over the row's G threads:
                 // the count is exact, the column is the row's only kept one when the count is 1
                 int pk = ((sizeof(Mask) == 8 ? __popcll((unsigned long long)bits) : __popc((unsigned)bits)) << 16) +
@@ -732,19 +916,20 @@ __global__ void __launch_bounds__(CH * G * G, blocks_for(CH * G * G, (int)sizeof
                 conv = __syncthreads_and(t > 0 && (!act || cnt == 1));
             }
 
+            bool requeue = false;  // Q gave way to the posteriors of forced convergence
             if (t > 0) {
                 bool have_cand = false, cand_forced = false;
                 int cand_p = -1;
                 if (conv) {
-                    any_conv = true;
+                    if (tid == 0) sh_flags |= F_CONVERGED;
                     have_cand = true;
                     cand_p = chosen;
                 } else if (a.decoder == 1 || t == a.T) {
                     // ---- forced convergence on lambda^t by locally dominant rounds
-                    forced_ran = true;
+                    if (tid == 0) sh_flags |= F_FORCED_RAN;
                     if (act && g == 0) matched[i] = 0;
                     __syncthreads();
-                    const T lii = act ? Lm[i * P + i] + Dg[i] : ninf;
+                    const T dgi = act ? Dg[i] : T(0);
                     if (a.forced_static) {
                         // the paper's static partition: row i's block is v_ik, k >= i; its
                         // maximum (ties: smaller k) represents factor i; representatives are
@@ -756,7 +941,7 @@ __global__ void __launch_bounds__(CH * G * G, blocks_for(CH * G * G, (int)sizeof
                             for (int c = 0; c < CH; ++c) {
                                 const int k = COL(c);
                                 if (k >= i && k < s) {
-                                    const T lam = k == i ? lii : RL(c) + (CM(c) + RM(c));
+                                    const T lam = k == i ? RL(c) + dgi : RL(c) + (CM(c) + RM(c));
                                     if (bk < 0 || lam > bl) {
                                         bl = lam;
                                         bk = k;
@@ -807,41 +992,54 @@ __global__ void __launch_bounds__(CH * G * G, blocks_for(CH * G * G, (int)sizeof
                         }
                         __syncthreads();
                     }
-                    for (int round = 0; round < s && !a.forced_static; ++round) {
-                        const bool open = act && !matched[i];
-                        T bl = ninf;
-                        int bk = -1;
-                        if (open) {
+                    // Rows choose their best unmatched column; a variable chosen by both its rows (or
+                    // the boundary) is accepted.  Unmatched rows are a bit set, columns are compared
+                    // without branches, and a row whose choice is still unmatched keeps it: the best
+                    // of a set that has only shrunk around it.
+                    if (!a.forced_static) {
+                        if (tid < (SMAX + 31) / 32) sh_open[tid] = s >= 32 * (tid + 1) ? kFull : s <= 32 * tid ? 0u : (1u << (s & 31)) - 1u;
+                        __syncthreads();
+                    }
+                    int ch = -1;
+                    if (!a.forced_static && act) {
+                        // the row's posteriors take the place of Q (read again if the shot goes on)
 #pragma unroll
-                            for (int c = 0; c < CH; ++c) {
-                                const int k = COL(c);
-                                if (k == i || !matched[k]) {
-                                    const T lam = k == i ? lii : RL(c) + (CM(c) + RM(c));
-                                    if (bk < 0 || lam > bl) {
-                                        bl = lam;
-                                        bk = k;
-                                    }
+                        for (int c = 0; c < CH; ++c) q[c] = COL(c) == i ? RL(c) + dgi : RL(c) + (CM(c) + RM(c));
+                    }
+                    requeue = !a.forced_static;
+                    for (int round = 0; round < s && !a.forced_static; ++round) {
+                        const bool open = act && ((sh_open[i >> 5] >> (i & 31)) & 1u);
+                        const bool scan = open && (round == 0 || !((sh_open[ch >> 5] >> (ch & 31)) & 1u));
+                        if (__any_sync(kFull, scan)) {
+                            T bl = ninf;
+                            int bk = -1;
+                            if (scan) {
+#pragma unroll
+                                for (int c = 0; c < CH; ++c) {
+                                    const int k = COL(c);
+                                    const bool up = ((sh_open[k >> 5] >> (k & 31)) & 1u) && (bk < 0 || q[c] > bl);
+                                    bl = up ? q[c] : bl;
+                                    bk = up ? k : bk;
                                 }
                             }
-                        }
 #pragma unroll
-                        for (int off = R; off < 32; off <<= 1) {
-                            const T ol = __shfl_xor_sync(kFull, bl, off);
-                            const int ok = __shfl_xor_sync(kFull, bk, off);
-                            if (ok >= 0 && (bk < 0 || ol > bl || (ol == bl && ok < bk))) {
-                                bl = ol;
-                                bk = ok;
+                            for (int off = R; off < 32; off <<= 1) {
+                                const T ol = __shfl_xor_sync(kFull, bl, off);
+                                const int ok = __shfl_xor_sync(kFull, bk, off);
+                                if (ok >= 0 && (bk < 0 || ol > bl || (ol == bl && ok < bk))) {
+                                    bl = ol;
+                                    bk = ok;
+                                }
+                            }
+                            if (scan) {
+                                ch = bk >= 0 ? bk : i;
+                                if (g == 0) choice[i] = ch;
                             }
                         }
-                        if (open && g == 0) choice[i] = bk >= 0 ? bk : i;
                         __syncthreads();
-                        bool newm = false;
-                        if (open && g == 0) {
-                            const int pk = choice[i];
-                            newm = (pk == i) || (choice[pk] == i);
-                        }
+                        const bool newm = open && (ch == i || choice[ch] == i);
                         __syncthreads();
-                        if (newm) matched[i] = 1;
+                        if (newm && g == 0) atomicAnd(&sh_open[i >> 5], ~(1u << (i & 31)));
                         const int left = __syncthreads_count(open && g == 0 && !newm);
                         if (tid == 0) acc_fcr += 1;
                         if (left == 0) break;
@@ -862,7 +1060,8 @@ __global__ void __launch_bounds__(CH * G * G, blocks_for(CH * G * G, (int)sizeof
                                 pc = Psh[i * SMAX + k];
                                 if (full) w = Wsh[i * SMAX + k];
                             } else {
-                                const size_t off = (size_t)dets[i] * n + dets[k];
+                                const ItemCtx ic = resolve_item(a, code);
+                                const size_t off = (size_t)dets[i] * ic.tb.n_det + dets[k];
                                 pc = ic.tb.P[off];
                                 if (full) w = ic.tb.W64[off];
                             }
@@ -874,6 +1073,7 @@ __global__ void __launch_bounds__(CH * G * G, blocks_for(CH * G * G, (int)sizeof
                     if (!full) {
                         out_par = par;
                         out_forced = cand_forced;
+                        out_from_best = 0;
                         partner = cand_p;
                         finish = true;
                     } else {
@@ -900,11 +1100,13 @@ __global__ void __launch_bounds__(CH * G * G, blocks_for(CH * G * G, (int)sizeof
                             if (a.decoder == 0 && cand_forced && !sh_use_best) {
                                 out_par = par;
                                 out_forced = 1;
+                                out_from_best = 0;
                                 partner = cand_p;
                             } else {
                                 out_par = sh_best_par;
                                 out_forced = sh_best_forced;
                                 out_from_best = 1;
+                                partner = -1;
                             }
                         }
                         __syncthreads();
@@ -913,79 +1115,21 @@ __global__ void __launch_bounds__(CH * G * G, blocks_for(CH * G * G, (int)sizeof
                 }
             }
 
-            // ---- compute phase: leave-one-out max* of every row, in place.  With m1 (at
-            // column am) and m2 the two largest Q of the row and S = sum_k 2^(min(Q_k, m2) - m2)
-            // (the max clamped to m2, so S - 1 = sum_{k != am} 2^(Q_k - m2) >= 1):
-            //   k != am: M'[i][k] = -(m1 + lg2(1 + 2^(m2 - m1) (S - 1 - 2^(Q_k - m2))))
-            //   k == am: M'[i][k] = -(m2 + lg2(S - 1))
-            // (the generic value is written for every column, the owner of am then overwrites;
-            // row i's outputs M'[i][k] go to Mt[k][i]).  FP32: (m1, m2, am) come from the read
-            // phase; FP64: from the scan below.
-            if (wact) {
+            // ---- compute phase, in place (FP64: the scan for (m1, m2, am) first)
+            if (requeue) {
                 if constexpr (std::is_same<T, float>::value) {
-                    const float2 nm2 = make_float2(-m2, -m2);
-                    float2 s2 = make_float2(0.f, 0.f);
+                    read_rows();
+                } else if (act) {
 #pragma unroll
-                    for (int j = 0; j < CH / 2; ++j) {
-                        const float2 dq = __fadd2_rn(q.p[j], nm2);
-                        const float2 u = make_float2(B2<float>::ex2(dq.x), B2<float>::ex2(dq.y));
-                        q.p[j] = u;
-                        s2 = __fadd2_rn(s2, make_float2(sat1(u.x), sat1(u.y)));
-                    }
-                    float S32 = s2.x + s2.y;
-#pragma unroll
-                    for (int off = R; off < 32; off <<= 1) S32 += __shfl_xor_sync(kFull, S32, off);
-                    const float cf32 = B2<float>::ex2(m2 - m1);
-                    const float Aa32 = __fmaf_rn(cf32, S32 - 1.f, 1.f);
-                    // 16-bit storage: this row's reference r_i = m1 rounded to the format (so
-                    // that it is exact there); stored values out + r_i = -lg2(Aa - cf u) + (r_i - m1)
-                    float rf32 = 0.f, dref32 = 0.f;
-                    if constexpr (HALF) {
-                        rf32 = IO::unpack(IO::pack(m1, 0.f)).x;
-                        dref32 = rf32 - m1;
-                    }
-                    if (act) {
-                        const float rf = rf32;
-                        // out = -m1 - lg2(Aa - cf u), the subtraction as an exact fma with -1
-                        const float2 ncf = make_float2(-cf32, -cf32), A2 = make_float2(Aa32, Aa32);
-                        const float2 nm1 = HALF ? make_float2(dref32, dref32) : make_float2(-m1, -m1);
-                        const float2 neg1 = make_float2(-1.f, -1.f);
-#pragma unroll
-                        for (int j = 0; j < CH / 2; ++j) {
-                            const float2 y = __ffma2_rn(ncf, q.p[j], A2);
-                            const float2 lg = make_float2(B2<float>::lg2(y.x), B2<float>::lg2(y.y));
-                            const float2 out = __ffma2_rn(lg, neg1, nm1);
-                            if constexpr (HALF) {
-                                // store the rounded pair (relative to r_i): both ends of a variable
-                                // read the same message
-                                const unsigned pk2 = IO::pack(out.x, out.y);
-                                *reinterpret_cast<unsigned short*>(CMP(2 * j)) = (unsigned short)(pk2 & 0xFFFFu);
-                                *reinterpret_cast<unsigned short*>(CMP(2 * j + 1)) = (unsigned short)(pk2 >> 16);
-                            } else {
-                                *CMP(2 * j) = out.x;
-                                *CMP(2 * j + 1) = out.y;
-                            }
-                        }
-                        if (own_max) {
-                            const float lgS = B2<float>::lg2(S32 - 1.f);
-                            if constexpr (HALF)
-                                IO::st(Mt + am * PM + i, __fmaf_rn(lgS, -1.f, rf - m2));
-                            else
-                                IO::st(Mt + am * PM + i, -m2 - lgS);
-                        }
-                        if (own_diag) {
-                            if constexpr (HALF) {
-                                // the diagonal holds r_i, which decodes to exactly 0
-                                Dg[i] = IO::ld(Mt + i * PM + i) + (-rf);
-                                IO::st(Mt + i * PM + i, rf);
-                                nrefv[i] = -rf;
-                            } else {
-                                Dg[i] = IO::ld(Mt + i * PM + i);
-                                Mt[i * PM + i] = MS(0.f);
-                            }
-                        }
-                    }
-                } else {
+                    for (int c = 0; c < CH; ++c) q[c] = B2<T>::fma_(RM(c), ainv, RL(c));
+                }
+                __syncthreads();
+            }
+            if constexpr (std::is_same<T, float>::value) {
+                update_rows();
+            } else {
+                if (wact) {
+                    int am = 0x7fffffff;
                     T a1 = ninf, a2 = ninf, b1 = ninf, b2 = ninf;
                     int ac = 0x7fffffff, bc = 0x7fffffff;
 #pragma unroll
@@ -1043,7 +1187,7 @@ __global__ void __launch_bounds__(CH * G * G, blocks_for(CH * G * G, (int)sizeof
                             *CMP(c) = out;
                         }
                         const T oam = -m2 - B2<T>::lg2(S - T(1));
-                        if (owner_of<PAIR, G>(am) == g) IO::st(Mt + am * PM + i, oam);
+                        if (owner_of<PAIR, G>(am) == g) Mt[am * PM + i] = oam;
                         if (own_diag) {
                             Dg[i] = IO::ld(Mt + i * PM + i);
                             Mt[i * PM + i] = MS(0.f);
@@ -1064,16 +1208,17 @@ __global__ void __launch_bounds__(CH * G * G, blocks_for(CH * G * G, (int)sizeof
             for (int k = s + tid; k < a.s_cap; k += NT) a.tr_partner[(size_t)shot * a.s_cap + k] = -1;
         }
         if (tid == 0) {
-            if (ic.obs_pred) ic.obs_pred[shot] = (uint8_t)out_par;
+            const ItemCtx ic = resolve_item(a, code);
+            if (ic.obs_pred) ic.obs_pred[ic.shot] = (uint8_t)out_par;
             if (ic.flags)
-                ic.flags[shot] = (uint8_t)((any_conv ? F_CONVERGED : 0) | (forced_ran ? F_FORCED_RAN : 0) |
-                                          (out_forced ? F_FROM_FORCED : 0));
-            if (ic.iters) ic.iters[shot] = (int16_t)t;
+                ic.flags[ic.shot] = (uint8_t)(sh_flags | (out_forced ? F_FROM_FORCED : 0));
+            if (ic.iters) ic.iters[ic.shot] = (int16_t)t;
             acc_it += (unsigned long long)t;
             acc_msg += (unsigned long long)s * s * t;
             acc_def += (unsigned long long)s;
             acc_shots += 1;
         }
+        if constexpr (HELP) pb ^= 1;
         __syncthreads();
     }
     if (tid == 0 && a.ctr) {
@@ -1117,10 +1262,11 @@ inline int64_t rw_slot_layout(int smax, int nt, int nodes) {
     return (b + 255) / 256 * 256;
 }
 
-template <typename T, int CH, int G, typename MS = T>
+template <typename T, int CH, int G, typename MS = T, bool RW = false>
 size_t smem_bytes_of() {
     constexpr int SMAX = CH * G;
-    return nref_offset<T, MS>(SMAX, G) + (sizeof(MS) == 2 ? (size_t)SMAX * sizeof(float) : 0) + (size_t)SMAX * 2 + 16;
+    return nref_offset<T, MS>(SMAX, G, helper_warp(SMAX, (int)sizeof(T), (int)sizeof(MS), RW)) +
+           (sizeof(MS) == 2 ? (size_t)SMAX * sizeof(float) : 0) + (size_t)SMAX * 2 + 16;
 }
 
 template <typename T, int CH, int G, bool TRACE, typename MS = T>
@@ -1130,10 +1276,11 @@ cudaError_t run_tier(const DecodeArgs& a, int num_sms, cudaStream_t st, bool pre
     if (prepare_only)
         return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     int per_sm = 0;
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, CH * G * G, smem);
+    constexpr int NT = block_threads(CH, G, (int)sizeof(T), (int)sizeof(MS), false);
+    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, NT, smem);
     if (e != cudaSuccess) return e;
     if (per_sm < 1) return cudaErrorInvalidConfiguration;
-    kern<<<per_sm * num_sms, CH * G * G, smem, st>>>(a);
+    kern<<<per_sm * num_sms, NT, smem, st>>>(a);
     return cudaGetLastError();
 }
 

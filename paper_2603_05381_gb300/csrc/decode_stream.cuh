@@ -99,16 +99,6 @@ template <typename T, int CH, typename MS, int CL = 1>
 constexpr int kStreamStages =
     stream_smem_bytes_n<T, CH, MS, CL>(2) <= (kStreamBlocks<T, CH, CL> == 2 ? 113u : 227u) * 1024u ? 2 : 1;
 
-// 16-byte asynchronous global->shared copies (cp.async, L2 only), used to fetch a warp's next
-// factor row while it works on the current one
-__device__ __forceinline__ void cp_async16(void* smem_dst, const void* gmem_src) {
-    const unsigned d = (unsigned)__cvta_generic_to_shared(smem_dst);
-    const size_t g = __cvta_generic_to_global(gmem_src);
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(g) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
-
 template <typename T>
 __device__ __forceinline__ T warp_max(T v) {
 #pragma unroll

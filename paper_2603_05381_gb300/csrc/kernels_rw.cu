@@ -15,7 +15,7 @@ namespace {
 template <typename T, int CH, int G>
 cudaError_t rw_grid(int n_det, int num_sms, int* grid, int64_t* slot_bytes, size_t* smem_out) {
     constexpr int SMAX = CH * G, NT = CH * G * G;
-    const size_t smem = smem_bytes_of<T, CH, G>();
+    const size_t smem = smem_bytes_of<T, CH, G, T, true>();
     auto kern = decode_smem_kernel<T, CH, G, false, true>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
