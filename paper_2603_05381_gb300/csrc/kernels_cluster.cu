@@ -1,6 +1,6 @@
 // Cluster form of the streaming tier: instantiations for FP32 messages and the choice of the
 // cluster size (kernels_cluster_half.cu holds the 16-bit message instantiations).
-#include "decode_stream.cuh"
+#include "decode_wide.cuh"
 
 namespace bp4m {
 
@@ -15,7 +15,7 @@ constexpr bool cl_f32(int ch, int cl) {
 template <int CH, int CL>
 cudaError_t launch_f32(const DecodeArgs& a, int slots, cudaStream_t st) {
     if constexpr (cl_f32(CH, CL))
-        return run_stream_cluster<float, CH, float, CL>(a, slots, st);
+        return run_wide_cluster<CH, float, CL>(a, slots, st);
     else
         return cudaErrorInvalidValue;
 }
@@ -23,7 +23,7 @@ cudaError_t launch_f32(const DecodeArgs& a, int slots, cudaStream_t st) {
 template <int CH, int CL>
 int capacity_f32() {
     if constexpr (cl_f32(CH, CL))
-        return stream_cluster_capacity<float, CH, float, CL>();
+        return wide_cluster_capacity<CH, float, CL>();
     else
         return 0;
 }
@@ -53,7 +53,7 @@ int capacity_f32_cl(int cl) {
 }  // namespace
 
 int stream_cluster_default(int ch) {
-    // Slots of all clusters in flight (16 B per element and LD^2 elements each in FP32) of
+    // Slots of all clusters in flight (12 B per element and LD^2 elements each in FP32) of
     // at most ~90 MB, so that they stay in the 126 MB L2 beside the other data.
     return ch <= 10 ? 4 : ch <= 14 ? 8 : 16;
 }

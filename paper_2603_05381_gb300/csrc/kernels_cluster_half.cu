@@ -1,6 +1,6 @@
 // Cluster form of the streaming tier with 16-bit message storage (precision 2 = IEEE half,
 // 3 = bfloat16): one cluster size per width, the default of stream_cluster_default().
-#include "decode_stream.cuh"
+#include "decode_wide.cuh"
 
 namespace bp4m {
 
@@ -11,13 +11,13 @@ constexpr int cl_half(int ch) { return ch <= 10 ? 4 : ch <= 14 ? 8 : 16; }
 template <typename MS, int CH>
 cudaError_t launch_h(int cl, const DecodeArgs& a, int slots, cudaStream_t st) {
     if (cl != cl_half(CH)) return cudaErrorInvalidValue;
-    return run_stream_cluster<float, CH, MS, cl_half(CH)>(a, slots, st);
+    return run_wide_cluster<CH, MS, cl_half(CH)>(a, slots, st);
 }
 
 template <typename MS, int CH>
 int capacity_h(int cl) {
     if (cl != cl_half(CH)) return 0;
-    return stream_cluster_capacity<float, CH, MS, cl_half(CH)>();
+    return wide_cluster_capacity<CH, MS, cl_half(CH)>();
 }
 
 template <typename MS>

@@ -11,6 +11,7 @@
 
 #include "decode_smem.cuh"
 #include "decode_stream.cuh"
+#include "decode_wide.cuh"
 #include "device.cuh"
 
 namespace bp4m {
@@ -548,7 +549,7 @@ int stream_cluster_for(int precision, int gsmax, int requested, int64_t shots, i
 
 int global_blocks_per_sm(int precision, int max_s) {
     const int ch = stream_ch(precision, max_s);
-    return (precision != 0 && ch != 0 && ch <= 8) ? kStreamBlocks<float, 8> : 1;
+    return precision != 0 && ch != 0 ? wide_blocks(ch, precision == 1 ? 4 : 2) : 1;
 }
 
 size_t global_slot_bytes(int precision, int max_s, int* gsmax_out) {
@@ -557,9 +558,9 @@ size_t global_slot_bytes(int precision, int max_s, int* gsmax_out) {
     if (ch) {
         const int ld = 32 * ch;
         *gsmax_out = ld;
-        return precision == 0   ? stream_slot_bytes<double, double>(ld)
-               : precision == 1 ? stream_slot_bytes<float, float>(ld)
-                                : stream_slot_bytes<float, __half>(ld);  // 16-bit messages, FP32 priors
+        return precision == 0   ? stream_slot_bytes(ld)
+               : precision == 1 ? wide_slot_bytes<float>(ld)
+                                : wide_slot_bytes<__half>(ld);  // 16-bit messages, FP32 priors
     }
     const int gsmax = (max_s + 63) / 64 * 64;
     *gsmax_out = gsmax;
@@ -577,20 +578,20 @@ cudaError_t launch_decode_global(int precision, const DecodeArgs& a, int slots, 
         }
         if (precision >= 2) return launch_stream_half(precision, ch, a, slots, st);
         if (precision == 0) {
-            if (ch == 8) return run_stream<double, 8>(a, slots, st);
-            return run_stream<double, 16>(a, slots, st);
+            if (ch == 8) return run_stream<8>(a, slots, st);
+            return run_stream<16>(a, slots, st);
         }
         switch (ch) {
-            case 6: return run_stream<float, 6>(a, slots, st);
-            case 8: return run_stream<float, 8>(a, slots, st);
-            case 10: return run_stream<float, 10>(a, slots, st);
-            case 12: return run_stream<float, 12>(a, slots, st);
-            case 14: return run_stream<float, 14>(a, slots, st);
-            case 16: return run_stream<float, 16>(a, slots, st);
-            case 20: return run_stream<float, 20>(a, slots, st);
-            case 24: return run_stream<float, 24>(a, slots, st);
-            case 28: return run_stream<float, 28>(a, slots, st);
-            default: return run_stream<float, 32>(a, slots, st);
+            case 6: return run_wide<6, float>(a, slots, st);
+            case 8: return run_wide<8, float>(a, slots, st);
+            case 10: return run_wide<10, float>(a, slots, st);
+            case 12: return run_wide<12, float>(a, slots, st);
+            case 14: return run_wide<14, float>(a, slots, st);
+            case 16: return run_wide<16, float>(a, slots, st);
+            case 20: return run_wide<20, float>(a, slots, st);
+            case 24: return run_wide<24, float>(a, slots, st);
+            case 28: return run_wide<28, float>(a, slots, st);
+            default: return run_wide<32, float>(a, slots, st);
         }
     }
     const size_t smem = global_kernel_smem(a.gsmax);

@@ -7,7 +7,7 @@
 #include <cuda_runtime.h>
 
 #include "decode_smem.cuh"
-#include "decode_stream.cuh"
+#include "decode_wide.cuh"
 #include "device.cuh"
 
 namespace bp4m {
@@ -31,16 +31,16 @@ cudaError_t dispatch_half(int tier, const DecodeArgs& a, int num_sms, cudaStream
 template <typename MS>
 cudaError_t dispatch_stream_half(int ch, const DecodeArgs& a, int slots, cudaStream_t st) {
     switch (ch) {
-        case 6: return run_stream<float, 6, MS>(a, slots, st);
-        case 8: return run_stream<float, 8, MS>(a, slots, st);
-        case 10: return run_stream<float, 10, MS>(a, slots, st);
-        case 12: return run_stream<float, 12, MS>(a, slots, st);
-        case 14: return run_stream<float, 14, MS>(a, slots, st);
-        case 16: return run_stream<float, 16, MS>(a, slots, st);
-        case 20: return run_stream<float, 20, MS>(a, slots, st);
-        case 24: return run_stream<float, 24, MS>(a, slots, st);
-        case 28: return run_stream<float, 28, MS>(a, slots, st);
-        case 32: return run_stream<float, 32, MS>(a, slots, st);
+        case 6: return run_wide<6, MS>(a, slots, st);
+        case 8: return run_wide<8, MS>(a, slots, st);
+        case 10: return run_wide<10, MS>(a, slots, st);
+        case 12: return run_wide<12, MS>(a, slots, st);
+        case 14: return run_wide<14, MS>(a, slots, st);
+        case 16: return run_wide<16, MS>(a, slots, st);
+        case 20: return run_wide<20, MS>(a, slots, st);
+        case 24: return run_wide<24, MS>(a, slots, st);
+        case 28: return run_wide<28, MS>(a, slots, st);
+        case 32: return run_wide<32, MS>(a, slots, st);
         default: return cudaErrorInvalidValue;
     }
 }
