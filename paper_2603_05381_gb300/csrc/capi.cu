@@ -81,8 +81,8 @@ struct Workspace {
     uint8_t* obs_pred = nullptr;
     uint8_t* flags = nullptr;
     int16_t* iters = nullptr;
-    int32_t* lists = nullptr;     // [kTiers][cap]
-    int32_t* small = nullptr;     // counts[kTiers], next[kTiers], max_s
+    int32_t* lists = nullptr;     // [kTiers][cap], two lists per slot (list_slot, list_back)
+    int32_t* small = nullptr;     // counts[kLists], next[kLists], max_s
     unsigned long long* ctr = nullptr;
     int32_t* host_small = nullptr;  // pinned mirror of `small`
     unsigned long long* host_ctr = nullptr;
@@ -150,6 +150,17 @@ int n_words_of(const bp4m_graph* g, int ty) { return (g->host.t[ty].n_det + 31) 
 
 enum { PROF_CLASSIFY = 0, PROF_GLOBAL = kGlobalTier, PROF_SAMPLE = kGlobalTier + 1, PROF_COUNT = kGlobalTier + 2 };
 static_assert(PROF_COUNT + 1 == BP4M_PROF_SLOTS, "profile slots");
+
+constexpr int kSmallInts = 2 * kLists + 1;  // counts[kLists], next[kLists], max_s
+
+// Points a launch at list c of a list storage of [kTiers][stride] with its counters in `small`.
+void use_list(DecodeArgs& a, const int32_t* lists, int64_t stride, int32_t* small, int c) {
+    a.list = lists + (int64_t)list_slot(c) * stride + (list_back(c) ? stride - 1 : 0);
+    a.list_dir = list_back(c) ? -1 : 1;
+    a.count = small + c;
+    a.next = small + kLists + c;
+    a.tier = list_tier(c);
+}
 
 // Brackets one kernel launch with events when profiling is on.
 struct ProfScope {
@@ -366,9 +377,9 @@ int ensure_ws(bp4m_graph* g, Workspace& w, int64_t cap) {
     CK(dalloc(&w.flags, (size_t)cap * nt));
     CK(dalloc(&w.iters, (size_t)cap * nt));
     CK(dalloc(&w.lists, (size_t)cap * kTiers));
-    CK(dalloc(&w.small, 2 * kTiers + 1));
+    CK(dalloc(&w.small, kSmallInts));
     CK(dalloc(&w.ctr, C_NUM));
-    CK(cudaMallocHost(reinterpret_cast<void**>(&w.host_small), (2 * kTiers + 1) * sizeof(int32_t)));
+    CK(cudaMallocHost(reinterpret_cast<void**>(&w.host_small), kSmallInts * sizeof(int32_t)));
     CK(cudaMallocHost(reinterpret_cast<void**>(&w.host_ctr), C_NUM * sizeof(unsigned long long)));
     CK(cudaEventCreateWithFlags(&w.ev_small, cudaEventDisableTiming));
     return BP4M_OK;
@@ -528,18 +539,21 @@ int decode_device(bp4m_graph* g, Workspace& w, int ty, const uint32_t* synd, int
         CK(prepare_decode_kernels(pio));
         g->prepared[pio] = true;
     }
-    const TierPlan plan = tier_plan(prec);
-    CK(cudaMemsetAsync(w.small, 0, (2 * kTiers + 1) * sizeof(int32_t), st));
+    const TierPlan plan = tier_plan(prec, rw != nullptr);
+    CK(cudaMemsetAsync(w.small, 0, kSmallInts * sizeof(int32_t), st));
     {
         ProfScope ps(g, PROF_CLASSIFY, st);
-        CK(launch_classify(synd, shots, n_words_of(g, ty), plan, w.lists, w.small, w.small + 2 * kTiers,
+        CK(launch_classify(synd, shots, n_words_of(g, ty), plan, w.lists, w.small, w.small + 2 * kLists,
                            obs_pred, flags, iters, tr ? tr->defects : nullptr, rw ? rw->skip : nullptr,
                            rw ? rw->skip_obs : nullptr, rw ? rw->skip_iters : nullptr, st));
         ps.end();
     }
-    CK(cudaMemcpyAsync(w.host_small, w.small, (2 * kTiers + 1) * sizeof(int32_t),
+    // the counts decide which lists are launched: a launch for an empty list costs about what
+    // the wait does, and most batches fill only a few of them
+    CK(cudaMemcpyAsync(w.host_small, w.small, kSmallInts * sizeof(int32_t),
                        cudaMemcpyDeviceToHost, st));
     CK(cudaEventRecord(w.ev_small, st));
+    CK(cudaEventSynchronize(w.ev_small));
     DecodeArgs a;
     a.tb = dev_tables(g, ty);
     a.synd = synd;
@@ -568,13 +582,13 @@ int decode_device(bp4m_graph* g, Workspace& w, int ty, const uint32_t* synd, int
         a.rw_off = g->rw_off[ty];
         a.rw_adj = g->rw_adj[ty];
         a.rw_units = g->host.n_units;
-        const int max_tier = prec == 0 ? kRwMaxTier64 : kRwMaxTier32;
-        // the tiers run one after another on `st` and share the scratch; each launch has
+        // the lists run one after another on `st` and share the scratch; each launch has
         // its own grid and slot size
         size_t need = 0;
-        int64_t slot[kTiers] = {};
-        for (int tier = 1; tier <= max_tier; ++tier) {
-            const size_t b = rw_scratch_bytes(prec, tier, g->host.t[ty].n_det, g->num_sms, &slot[tier]);
+        int64_t slot[kLists] = {};
+        for (int c = 0; c < kGlobalList; ++c) {
+            if (!plan.used(c)) continue;
+            const size_t b = rw_scratch_bytes(prec, c, g->host.t[ty].n_det, g->num_sms, &slot[c]);
             if (b == 0) return fail(BP4M_ECUDA, "B-BP4MF: no launch configuration for a reweighting tier");
             need = std::max(need, b);
         }
@@ -582,36 +596,31 @@ int decode_device(bp4m_graph* g, Workspace& w, int ty, const uint32_t* synd, int
         if (rc) return rc;
         a.gscratch = w.gscratch;
         a.gscratch_bytes = (int64_t)w.gscratch_bytes;
-        for (int tier = 1; tier <= max_tier; ++tier) {
-            a.rw_slot_bytes = slot[tier];
-            a.list = w.lists + (size_t)tier * shots;
-            a.count = w.small + tier;
-            a.next = w.small + kTiers + tier;
-            a.tier = tier;
-            ProfScope ps(g, tier, st);
-            CK(launch_decode_tier_rw(prec, tier, a, g->num_sms, st));
+        for (int c = 0; c < kGlobalList; ++c) {
+            if (w.host_small[c] <= 0) continue;
+            a.rw_slot_bytes = slot[c];
+            use_list(a, w.lists, shots, w.small, c);
+            a.max_items = w.host_small[c];
+            ProfScope ps(g, a.tier, st);
+            CK(launch_decode_list_rw(prec, c, a, g->num_sms, st));
             ps.end();
         }
-        CK(cudaEventSynchronize(w.ev_small));
-        for (int tier = max_tier + 1; tier < kTiers; ++tier)
-            if (w.host_small[tier] > 0)
-                return fail(BP4M_EUNSUPPORTED, prec == 0 ? "B-BP4MF (FP64) decodes at most 112 unsatisfied checks of a type per shot"
-                                                         : "B-BP4MF (FP32) decodes at most 160 unsatisfied checks of a type per shot");
+        if (w.host_small[kGlobalList] > 0)
+            return fail(BP4M_EUNSUPPORTED, prec == 0 ? "B-BP4MF (FP64) decodes at most 112 unsatisfied checks of a type per shot"
+                                                     : "B-BP4MF (FP32) decodes at most 160 unsatisfied checks of a type per shot");
         return BP4M_OK;
     }
-    for (int tier = 1; tier < kGlobalTier; ++tier) {
-        a.list = w.lists + (size_t)tier * shots;
-        a.count = w.small + tier;
-        a.next = w.small + kTiers + tier;
-        a.tier = tier;
-        ProfScope ps(g, tier, st);
-        CK(launch_decode_tier(pio, tier, a, g->num_sms, st));
+    for (int c = 0; c < kGlobalList; ++c) {
+        if (w.host_small[c] <= 0) continue;
+        use_list(a, w.lists, shots, w.small, c);
+        a.max_items = w.host_small[c];
+        ProfScope ps(g, a.tier, st);
+        CK(launch_decode_list(pio, c, a, g->num_sms, st));
         ps.end();
     }
-    CK(cudaEventSynchronize(w.ev_small));
-    const int n_glob = w.host_small[kGlobalTier];
+    const int n_glob = w.host_small[kGlobalList];
     if (n_glob > 0) {
-        const int max_s = w.host_small[2 * kTiers];
+        const int max_s = w.host_small[2 * kLists];
         // width classes up to the batch's largest defect count; the scratch holds a slot for
         // every resident block of the class that needs most, whatever this batch's count, so
         // that it is reallocated (a device-wide synchronisation) only for a wider slot
@@ -622,15 +631,13 @@ int decode_device(bp4m_graph* g, Workspace& w, int ty, const uint32_t* synd, int
             rc = ensure_split(w, shots);
             if (rc) return rc;
         }
-        a.list = w.lists + (size_t)kGlobalTier * shots;
-        a.count = w.small + kGlobalTier;
+        use_list(a, w.lists, shots, w.small, kGlobalList);
         a.gscratch = w.gscratch;
         a.gscratch_bytes = (int64_t)w.gscratch_bytes;
-        a.tier = kGlobalTier;
         ProfScope ps(g, PROF_GLOBAL, st);
         if (p.gc.n == 1) {
             a.stream_cl = stream_cluster_for(pio, p.gsmax[0], o->stream_cluster, n_glob, p.full[0]);
-            rc = launch_global_classes(a, p, pio, n_glob, w.sub, w.subctr, shots, w.small + kTiers + kGlobalTier,
+            rc = launch_global_classes(a, p, pio, n_glob, w.sub, w.subctr, shots, w.small + kLists + kGlobalList,
                                        g->num_sms, st);
             if (rc) return rc;
         } else {
@@ -1170,13 +1177,13 @@ struct MultiHostEntry {
     uint8_t* h_out = nullptr;     // pinned [2][cap]: obs, flags
 };
 
-// Candidate tier plans of the autotuner, as the largest row count each FP32 tier takes;
-// a tier whose bound equals the previous one's is never populated.
+// Candidate list plans of the autotuner, as the largest row count each list takes; a list whose
+// bound equals the previous one's is never populated.
 constexpr int kPlanCount = 3;
-const int kPlanSmax[kPlanCount][kGlobalTier] = {
-    {0, 32, 64, 96, 112, 128, 144, 160},   // every tier (finest padding)
-    {0, 32, 64, 96, 96, 128, 128, 160},    // 32-row steps above 64
-    {0, 32, 64, 64, 112, 112, 144, 160},   // 48/32-row steps
+const int kPlanSmax[kPlanCount][kGlobalList] = {
+    {8, 16, 24, 32, 48, 64, 80, 96, 112, 128, 144, 160},   // every list (finest padding)
+    {8, 16, 24, 32, 32, 64, 64, 96, 96, 128, 128, 160},    // 32-row steps above 32
+    {8, 16, 24, 32, 32, 64, 64, 64, 112, 112, 144, 160},   // 48/32-row steps
 };
 
 }  // namespace
@@ -1192,7 +1199,7 @@ struct bp4m_multi {
     int64_t total_cap = 0;
     MultiEntry* d_entries = nullptr;
     int32_t* lists = nullptr;
-    int32_t* small = nullptr;          // counts[kTiers], next[kTiers], max_s
+    int32_t* small = nullptr;          // counts[kLists], next[kLists], max_s
     unsigned long long* ctr = nullptr;
     unsigned long long* h_ctr = nullptr;
     void* gscratch = nullptr;
@@ -1243,14 +1250,14 @@ int multi_enqueue(bp4m_multi* m, const std::vector<int64_t>& shots, int plan, in
         if (shots[k] > 0)
             CK(cudaMemcpyAsync(x.d_synd, x.h_synd, (size_t)shots[k] * x.n_words * 4, cudaMemcpyHostToDevice, st));
     }
-    CK(cudaMemsetAsync(m->small, 0, (2 * kTiers + 1) * sizeof(int32_t), st));
+    CK(cudaMemsetAsync(m->small, 0, kSmallInts * sizeof(int32_t), st));
     CK(cudaMemsetAsync(m->ctr, 0, C_NUM * sizeof(unsigned long long), st));
     TierPlan tp{};
-    for (int t = 0; t < kGlobalTier; ++t) tp.smax[t] = m->pio == 0 ? tier_plan(0).smax[t] : kPlanSmax[plan][t];
-    tp.smax[kGlobalTier] = 0x7fffffff;
+    for (int c = 0; c < kGlobalList; ++c) tp.smax[c] = m->pio == 0 ? tier_plan(0).smax[c] : kPlanSmax[plan][c];
+    tp.smax[kGlobalList] = 0x7fffffff;
     for (int k = 0; k < n; ++k) {
         const MultiHostEntry& x = m->e[k];
-        CK(launch_classify(x.d_synd, shots[k], x.n_words, tp, m->lists, m->small, m->small + 2 * kTiers, x.d_obs,
+        CK(launch_classify(x.d_synd, shots[k], x.n_words, tp, m->lists, m->small, m->small + 2 * kLists, x.d_obs,
                            x.d_flags, x.d_iters, nullptr, nullptr, nullptr, nullptr, st, m->total_cap,
                            (int32_t)((int64_t)k << kMultiShift)));
     }
@@ -1264,23 +1271,18 @@ int multi_enqueue(bp4m_multi* m, const std::vector<int64_t>& shots, int plan, in
     a.stream_cl = stream_cl;
     a.alpha = m->opts.alpha;
     a.ctr = m->ctr;
-    for (int tier = 1; tier < kGlobalTier; ++tier) {
-        if (m->pio != 0 && tier > 1 && kPlanSmax[plan][tier] == kPlanSmax[plan][tier - 1]) continue;
-        a.list = m->lists + (size_t)tier * m->total_cap;
-        a.count = m->small + tier;
-        a.next = m->small + kTiers + tier;
-        a.tier = tier;
-        CK(launch_decode_tier(m->pio, tier, a, m->num_sms, st));
+    for (int c = 0; c < kGlobalList; ++c) {
+        if (!tp.used(c)) continue;
+        use_list(a, m->lists, m->total_cap, m->small, c);
+        CK(launch_decode_list(m->pio, c, a, m->num_sms, st));
     }
-    a.list = m->lists + (size_t)kGlobalTier * m->total_cap;
-    a.count = m->small + kGlobalTier;
-    a.tier = kGlobalTier;
+    use_list(a, m->lists, m->total_cap, m->small, kGlobalList);
     a.gscratch = m->gscratch;
     {
         // every width class up to max_defects: the counts stay on the device
         const GlobalPlan p = global_plan(m->pio, m->max_defects, m->num_sms);
         const int rc = launch_global_classes(a, p, m->pio, m->total_cap, m->sub, m->subctr, m->total_cap,
-                                             m->small + kTiers + kGlobalTier, m->num_sms, st);
+                                             m->small + kLists + kGlobalList, m->num_sms, st);
         if (rc) return rc;
     }
     for (int k = 0; k < n; ++k) {
@@ -1529,7 +1531,7 @@ bp4m_multi* bp4m_multi_create(int n, bp4m_graph* const* graphs, const int* types
         }
     }
     if (dalloc(&m->d_entries, (size_t)n) != cudaSuccess || dalloc(&m->lists, (size_t)m->total_cap * kTiers) != cudaSuccess ||
-        dalloc(&m->small, 2 * kTiers + 1) != cudaSuccess || dalloc(&m->ctr, C_NUM) != cudaSuccess ||
+        dalloc(&m->small, kSmallInts) != cudaSuccess || dalloc(&m->ctr, C_NUM) != cudaSuccess ||
         cudaMallocHost(reinterpret_cast<void**>(&m->h_ctr), C_NUM * sizeof(unsigned long long)) != cudaSuccess)
         return bad(fail(BP4M_ENOMEM, "out of memory for the fused decode's lists"));
     if (cudaMemcpy(m->d_entries, host.data(), sizeof(MultiEntry) * n, cudaMemcpyHostToDevice) != cudaSuccess)

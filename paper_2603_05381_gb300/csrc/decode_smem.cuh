@@ -441,7 +441,7 @@ __global__ void __launch_bounds__(block_threads(CH, G, (int)sizeof(T), (int)size
         item = __shfl_sync(kFull, item, 0);
         int c = -1, s0 = 0;
         if (item < count) {
-            c = a.list[item];
+            c = a.list[(int64_t)item * a.list_dir];
             const ItemCtx ic = resolve_item(a, c);
             s0 = compact_defects(ic.synd + (size_t)ic.shot * ic.tb.n_words, ic.tb.n_words, dets0 + b * SMAX, SMAX, lane);
         }
@@ -470,7 +470,7 @@ __global__ void __launch_bounds__(block_threads(CH, G, (int)sizeof(T), (int)size
             __syncthreads();
             const int item = sh_item;
             if (item >= count) break;
-            code = a.list[item];
+            code = a.list[(int64_t)item * a.list_dir];
             if (warp == 0) {
                 const ItemCtx ic = resolve_item(a, code);
                 const int s0 = compact_defects(ic.synd + (size_t)ic.shot * ic.tb.n_words, ic.tb.n_words, dets, SMAX, lane);
@@ -1241,19 +1241,13 @@ __global__ void __launch_bounds__(block_threads(CH, G, (int)sizeof(T), (int)size
 
 // ------------------------------------------------------------------ tier table
 
-struct TierCfg {
-    int smax;
-    int ch, g;
-};
+// Row counts of the lists (0: not used).  FP32: 8..32 several shots per warp (decode_small.cuh),
+// 48..160 one shot per block; FP64 and the FP32 reweighting decode: coarser.  The 16-row steps
+// above 32 follow the defect counts (d = 13 circuit shots at p = 0.005: s = 126 +- 16).
+constexpr int kRows32[kGlobalList] = {8, 16, 24, 32, 48, 64, 80, 96, 112, 128, 144, 160};
+constexpr int kRowsRw32[kGlobalList] = {0, 0, 0, 32, 0, 64, 0, 96, 112, 128, 144, 160};
+constexpr int kRows64[kGlobalList] = {0, 0, 0, 32, 0, 64, 0, 0, 112, 0, 0, 0};
 
-// FP32: 32/64/96/112/128/144/160 rows in shared memory; FP64: 32/64/112 (tiers 4..7
-// unused).  The 16-row steps from 96 rows up follow the defect counts of circuit-level
-// shots (d = 13, p = 0.005: s = 126 +- 16), where padding rows and columns cost issue slots.
-constexpr int kSmemTiers = 7;
-constexpr TierCfg kCfg32[kSmemTiers + 1] = {{0, 0, 0},     {32, 32, 1},  {64, 32, 2},  {96, 24, 4},
-                                            {112, 28, 4}, {128, 32, 4}, {144, 36, 4}, {160, 40, 4}};
-constexpr TierCfg kCfg64[kSmemTiers + 1] = {{0, 0, 0},     {32, 16, 2},  {64, 16, 4},  {112, 28, 4},
-                                            {112, 28, 4}, {112, 28, 4}, {112, 28, 4}, {112, 28, 4}};
 // Bytes of one RW scratch slot: W [SMAX][SMAX] doubles, Dijkstra distances [warps][nodes]
 // doubles, parity [SMAX][SMAX] bytes, done and parity flags [warps][nodes] bytes.
 inline int64_t rw_slot_layout(int smax, int nt, int nodes) {
@@ -1269,18 +1263,38 @@ size_t smem_bytes_of() {
            (sizeof(MS) == 2 ? (size_t)SMAX * sizeof(float) : 0) + (size_t)SMAX * 2 + 16;
 }
 
+// Resident blocks per SM of a kernel on the current device, asked for once per kernel and device.
+constexpr int kOccDevices = 16;
+template <typename K>
+cudaError_t resident_blocks(K kern, int threads, size_t smem, std::atomic<int>* cache, int* per_sm) {
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev >= 0 && dev < kOccDevices && (*per_sm = cache[dev].load()) > 0) return cudaSuccess;
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, kern, threads, smem);
+    if (e != cudaSuccess) return e;
+    if (*per_sm < 1) return cudaErrorInvalidConfiguration;
+    if (dev >= 0 && dev < kOccDevices) cache[dev].store(*per_sm);
+    return cudaSuccess;
+}
+
+// Grid of a persistent launch: every resident block, or one per item where the items are fewer.
+inline int persistent_grid(int resident, const DecodeArgs& a) {
+    return a.max_items > 0 && a.max_items < resident ? (int)a.max_items : resident;
+}
+
 template <typename T, int CH, int G, bool TRACE, typename MS = T>
 cudaError_t run_tier(const DecodeArgs& a, int num_sms, cudaStream_t st, bool prepare_only) {
     const size_t smem = smem_bytes_of<T, CH, G, MS>();
     auto kern = decode_smem_kernel<T, CH, G, TRACE, false, MS>;
     if (prepare_only)
         return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    int per_sm = 0;
     constexpr int NT = block_threads(CH, G, (int)sizeof(T), (int)sizeof(MS), false);
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, NT, smem);
+    static std::atomic<int> cache[kOccDevices] = {};
+    int per_sm = 0;
+    cudaError_t e = resident_blocks(kern, NT, smem, cache, &per_sm);
     if (e != cudaSuccess) return e;
-    if (per_sm < 1) return cudaErrorInvalidConfiguration;
-    kern<<<per_sm * num_sms, NT, smem, st>>>(a);
+    kern<<<persistent_grid(per_sm * num_sms, a), NT, smem, st>>>(a);
     return cudaGetLastError();
 }
 

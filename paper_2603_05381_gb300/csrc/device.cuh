@@ -63,17 +63,32 @@ enum : uint8_t { F_CONVERGED = 1, F_FORCED_RAN = 2, F_FROM_FORCED = 4, F_FROM_QB
 constexpr int kTiers = 9;      // tier 0: s == 0 (done in classify), 1..7 shared memory, 8 global
 constexpr int kGlobalTier = 8;
 
+// Decode lists: the shots of a batch by defect count, finer than the tiers (padding rows and
+// columns cost issue slots).  Lists 0..3 (8, 16, 24, 32 rows) make up tier 1, 4 and 5 (48, 64)
+// tier 2, 6 and 7 (80, 96) tier 3, 8..11 are tiers 4..7 and 12 the global tier.  Two lists share
+// one slot of the list storage ([kTiers][cap]) from both ends, so the finer lists take no more
+// memory than one list per tier.
+constexpr int kLists = 13;
+constexpr int kGlobalList = 12;
+__host__ __device__ constexpr int list_slot(int c) { return c < 8 ? c >> 1 : c - 4; }
+__host__ __device__ constexpr bool list_back(int c) { return c < 8 && (c & 1) != 0; }
+__host__ __device__ constexpr int list_tier(int c) { return c < 4 ? 1 : c < 6 ? 2 : c < 8 ? 3 : c - 4; }
+
 struct TierPlan {
-    int smax[kTiers];  // inclusive upper bound of s for the tier (global tier: unbounded)
+    int smax[kLists];  // inclusive upper bound of s for the list (a list whose bound equals the
+                       // one before is never populated; global list: unbounded)
+    bool used(int c) const { return smax[c] > (c ? smax[c - 1] : 0); }
 };
 
 struct DecodeArgs {
     DevTables tb;
     const uint32_t* synd = nullptr;  // [shots][n_words]
     int64_t shots = 0;
-    const int32_t* list = nullptr;   // this tier's shot indices
+    const int32_t* list = nullptr;   // this list's shot indices, item k at list[k * list_dir]
+    int list_dir = 1;
     const int32_t* count = nullptr;  // number of entries in `list`
     int32_t* next = nullptr;         // work-stealing counter
+    int64_t max_items = 0;           // entries of `list` where the host knows them (bounds the grid), 0: unknown
     int T = 0;
     int early_exit = 1;
     int decoder = 0;                 // 0 = BP4M, 1 = BP4MF
@@ -203,11 +218,12 @@ cudaError_t launch_sample_circuit(const SampleArgs& a, cudaStream_t st);
 cudaError_t launch_sample_code_capacity(const SampleArgs& a, cudaStream_t st);
 
 // classify: per shot s = popcount; s == 0 results are written directly; the others are
-// appended to their tier's list.  counts[kTiers], max_s (int) must be zeroed before.
+// appended to their list (list c in slot list_slot(c) of `lists`, from the front or, with
+// list_back(c), from the back).  counts[kLists], max_s (int) must be zeroed before.
 // With `skip` (per-shot flag) non-null, flagged shots are not decoded: their outputs are
 // taken from skip_obs (the first stage of B-BP4MF) and skip_iters.
 cudaError_t launch_classify(const uint32_t* synd, int64_t shots, int n_words,
-                            const TierPlan& plan, int32_t* lists /*[kTiers][shots]*/,
+                            const TierPlan& plan, int32_t* lists /*[kTiers][list_stride]*/,
                             int32_t* counts, int32_t* max_s, uint8_t* obs_pred, uint8_t* flags,
                             int16_t* iters, int32_t* tr_defects, const uint8_t* skip,
                             const uint8_t* skip_obs, const int16_t* skip_iters, cudaStream_t st,
@@ -215,25 +231,27 @@ cudaError_t launch_classify(const uint32_t* synd, int64_t shots, int n_words,
 
 // Register-tile form of the FP32 shared-memory tiers (decode_reg.cuh): tiers that have one,
 // and its launch (or, with prepare_only, its one-time kernel attributes).
-bool reg_tier_available(int tier);
-cudaError_t launch_decode_tier_reg(int tier, const DecodeArgs& a, int num_sms, cudaStream_t st, bool prepare_only);
+bool reg_list_available(int list);
+cudaError_t launch_decode_list_reg(int list, const DecodeArgs& a, int num_sms, cudaStream_t st, bool prepare_only);
 // 16-bit message storage (precision 2 = IEEE half, 3 = bfloat16) of the shared-memory tiers.
-cudaError_t launch_decode_tier_half(int precision, int tier, const DecodeArgs& a, int num_sms, cudaStream_t st,
+cudaError_t launch_decode_list_half(int precision, int list, const DecodeArgs& a, int num_sms, cudaStream_t st,
                                     bool prepare_only);
-// Launch the decoding kernel of shared-memory tier `tier` (1..7) for precision
-// (0 = FP64, 1 = FP32).  Returns cudaSuccess if the tier is empty by construction.
-cudaError_t launch_decode_tier(int precision, int tier, const DecodeArgs& a, int num_sms,
+// Small shots, several per warp (decode_small.cuh): lists 0..3 with FP32 arithmetic (precision
+// 1 = FP32, 2 = IEEE half, 3 = bfloat16 messages).
+constexpr int kSmallLists = 4;
+cudaError_t launch_decode_small(int precision, int list, const DecodeArgs& a, int num_sms, cudaStream_t st,
+                                bool prepare_only);
+// Launch the decoding kernel of list `list` (0 .. kGlobalList - 1) for a precision (0 = FP64,
+// 1 = FP32, 2 and 3 = 16-bit messages); the list must be used by the precision's plan.
+cudaError_t launch_decode_list(int precision, int list, const DecodeArgs& a, int num_sms,
                                cudaStream_t st);
-// Reweighting (B-BP4MF second stage) decode of the shared-memory tiers (FP32 1..7, FP64
-// 1..3).  rw_scratch_bytes() is the global scratch the launch of `tier` needs for a graph
+// Reweighting (B-BP4MF second stage) decode of the lists that its plan (tier_plan with `rw`)
+// uses.  rw_scratch_bytes() is the global scratch the launch of a list needs for a graph
 // of n_det detectors (one slot per resident block) and sets *slot_bytes; the caller
 // passes that scratch in a.gscratch and the slot size in a.rw_slot_bytes.
-size_t rw_scratch_bytes(int precision, int tier, int n_det, int num_sms, int64_t* slot_bytes);
-cudaError_t launch_decode_tier_rw(int precision, int tier, const DecodeArgs& a, int num_sms,
+size_t rw_scratch_bytes(int precision, int list, int n_det, int num_sms, int64_t* slot_bytes);
+cudaError_t launch_decode_list_rw(int precision, int list, const DecodeArgs& a, int num_sms,
                                   cudaStream_t st);
-// Highest shared-memory tier per precision (FP64 tiers 4..7 are never populated).
-constexpr int kRwMaxTier32 = 7;
-constexpr int kRwMaxTier64 = 3;
 // Smallest edge weight of the reweighted graph: posteriors at or above one half would give
 // weights <= 0, for which shortest paths do not exist on an undirected graph.
 constexpr double kRwMinWeight = 9.5367431640625e-07;  // 2^-20
@@ -280,8 +298,8 @@ GlobalClasses global_classes(int precision, int max_s);
 // last bound goes to the last class.  max_items bounds a.count (sizes the grid).
 cudaError_t launch_partition_global(const DecodeArgs& a, const GlobalClasses& gc, int32_t* sub, int64_t stride,
                                     int32_t* sub_counts, int64_t max_items, int num_sms, cudaStream_t st);
-// Shared-memory tier plan for a precision.
-TierPlan tier_plan(int precision);
+// List plan for a precision; with `rw` the coarser one of the reweighting decode.
+TierPlan tier_plan(int precision, bool rw = false);
 cudaError_t prepare_decode_kernels(int precision);
 
 // Decodes shots 0 .. shots-1 with the global-memory kernel using the library's file-scope

@@ -379,72 +379,70 @@ static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoAllocBytes];
 constexpr int kMaxDevices = 64;
 std::atomic<void*> g_noalloc_addr[kMaxDevices];
 
-template <typename T>
-cudaError_t dispatch_tier(int tier, const DecodeArgs& a, int num_sms, cudaStream_t st, bool prep);
-
-// Form of the FP32 tiers that have both when the caller leaves the choice to the library
+// Form of the FP32 lists that have both when the caller leaves the choice to the library
 constexpr bool kRegTilesDefault = false;
 
-template <>
-cudaError_t dispatch_tier<float>(int tier, const DecodeArgs& a, int num_sms, cudaStream_t st, bool prep) {
-    // the register-tile form where the tier has one (both forms are prepared)
-    if (reg_tier_available(tier)) {
+cudaError_t dispatch_list32(int list, const DecodeArgs& a, int num_sms, cudaStream_t st, bool prep) {
+    if (list < kSmallLists) return launch_decode_small(1, list, a, num_sms, st, prep);
+    // the register-tile form where the list has one (both forms are prepared)
+    if (reg_list_available(list)) {
         if (prep) {
-            cudaError_t e = launch_decode_tier_reg(tier, a, num_sms, st, true);
+            cudaError_t e = launch_decode_list_reg(list, a, num_sms, st, true);
             if (e != cudaSuccess) return e;
         } else if (a.tile_form == 2 || (a.tile_form == 0 && kRegTilesDefault)) {
-            return launch_decode_tier_reg(tier, a, num_sms, st, false);
+            return launch_decode_list_reg(list, a, num_sms, st, false);
         }
     }
-    switch (tier) {
-        case 1: return run_tier2<float, 32, 1>(a, num_sms, st, prep);
-        case 2: return run_tier2<float, 32, 2>(a, num_sms, st, prep);
-        case 3: return run_tier2<float, 24, 4>(a, num_sms, st, prep);
-        case 4: return run_tier2<float, 28, 4>(a, num_sms, st, prep);
-        case 5: return run_tier2<float, 32, 4>(a, num_sms, st, prep);
-        case 6: return run_tier2<float, 36, 4>(a, num_sms, st, prep);
-        case 7: return run_tier2<float, 40, 4>(a, num_sms, st, prep);
+    switch (list) {
+        case 4: return run_tier2<float, 24, 2>(a, num_sms, st, prep);
+        case 5: return run_tier2<float, 32, 2>(a, num_sms, st, prep);
+        case 6: return run_tier2<float, 20, 4>(a, num_sms, st, prep);
+        case 7: return run_tier2<float, 24, 4>(a, num_sms, st, prep);
+        case 8: return run_tier2<float, 28, 4>(a, num_sms, st, prep);
+        case 9: return run_tier2<float, 32, 4>(a, num_sms, st, prep);
+        case 10: return run_tier2<float, 36, 4>(a, num_sms, st, prep);
+        case 11: return run_tier2<float, 40, 4>(a, num_sms, st, prep);
         default: return cudaErrorInvalidValue;
     }
 }
 
-template <>
-cudaError_t dispatch_tier<double>(int tier, const DecodeArgs& a, int num_sms, cudaStream_t st, bool prep) {
-    switch (tier) {
-        case 1: return run_tier2<double, 16, 2>(a, num_sms, st, prep);
-        case 2: return run_tier2<double, 16, 4>(a, num_sms, st, prep);
-        case 3: return run_tier2<double, 28, 4>(a, num_sms, st, prep);
-        case 4: case 5: case 6: case 7: return cudaSuccess;  // same bound as tier 3: never populated
+cudaError_t dispatch_list64(int list, const DecodeArgs& a, int num_sms, cudaStream_t st, bool prep) {
+    switch (list) {
+        case 3: return run_tier2<double, 16, 2>(a, num_sms, st, prep);
+        case 5: return run_tier2<double, 16, 4>(a, num_sms, st, prep);
+        case 8: return run_tier2<double, 28, 4>(a, num_sms, st, prep);
         default: return cudaErrorInvalidValue;
     }
 }
 
 }  // namespace
 
-TierPlan tier_plan(int precision) {
+TierPlan tier_plan(int precision, bool rw) {
+    const int* rows = precision == 0 ? kRows64 : rw ? kRowsRw32 : kRows32;
     TierPlan p{};
-    const TierCfg* c = precision == 0 ? kCfg64 : kCfg32;
-    for (int k = 0; k < kGlobalTier; ++k) p.smax[k] = c[k].smax;
-    p.smax[kGlobalTier] = 0x7fffffff;
+    for (int c = 0; c < kGlobalList; ++c) p.smax[c] = std::max(rows[c], c ? p.smax[c - 1] : 0);
+    p.smax[kGlobalList] = 0x7fffffff;
     return p;
+}
+
+cudaError_t launch_decode_list(int precision, int list, const DecodeArgs& a, int num_sms,
+                               cudaStream_t st) {
+    if (precision >= 2) return launch_decode_list_half(precision, list, a, num_sms, st, false);
+    return precision == 0 ? dispatch_list64(list, a, num_sms, st, false)
+                          : dispatch_list32(list, a, num_sms, st, false);
 }
 
 cudaError_t prepare_decode_kernels(int precision) {
     DecodeArgs dummy;
-    for (int tier = 1; tier < kGlobalTier; ++tier) {
-        cudaError_t e = precision == 0   ? dispatch_tier<double>(tier, dummy, 0, 0, true)
-                        : precision == 1 ? dispatch_tier<float>(tier, dummy, 0, 0, true)
-                                         : launch_decode_tier_half(precision, tier, dummy, 0, 0, true);
+    const TierPlan plan = tier_plan(precision);
+    for (int list = 0; list < kGlobalList; ++list) {
+        if (!plan.used(list)) continue;
+        cudaError_t e = precision == 0   ? dispatch_list64(list, dummy, 0, 0, true)
+                        : precision == 1 ? dispatch_list32(list, dummy, 0, 0, true)
+                                         : launch_decode_list_half(precision, list, dummy, 0, 0, true);
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
-}
-
-cudaError_t launch_decode_tier(int precision, int tier, const DecodeArgs& a, int num_sms,
-                               cudaStream_t st) {
-    if (precision >= 2) return launch_decode_tier_half(precision, tier, a, num_sms, st, false);
-    return precision == 0 ? dispatch_tier<double>(tier, a, num_sms, st, false)
-                          : dispatch_tier<float>(tier, a, num_sms, st, false);
 }
 
 int noalloc_max_defects() { return kNoAllocMaxDefects; }

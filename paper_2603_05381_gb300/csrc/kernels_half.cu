@@ -14,16 +14,17 @@ namespace bp4m {
 namespace {
 
 template <typename MS>
-cudaError_t dispatch_half(int tier, const DecodeArgs& a, int num_sms, cudaStream_t st, bool prep) {
-    switch (tier) {
-        case 1: return run_tier2<float, 32, 1, MS>(a, num_sms, st, prep);
-        case 2: return run_tier2<float, 32, 2, MS>(a, num_sms, st, prep);
-        case 3: return run_tier2<float, 24, 4, MS>(a, num_sms, st, prep);
-        case 4: return run_tier2<float, 28, 4, MS>(a, num_sms, st, prep);
+cudaError_t dispatch_half(int list, const DecodeArgs& a, int num_sms, cudaStream_t st, bool prep) {
+    switch (list) {
+        case 4: return run_tier2<float, 24, 2, MS>(a, num_sms, st, prep);
+        case 5: return run_tier2<float, 32, 2, MS>(a, num_sms, st, prep);
+        case 6: return run_tier2<float, 20, 4, MS>(a, num_sms, st, prep);
+        case 7: return run_tier2<float, 24, 4, MS>(a, num_sms, st, prep);
+        case 8: return run_tier2<float, 28, 4, MS>(a, num_sms, st, prep);
         // 128 rows: two blocks per SM
-        case 5: return run_tier2<float, 32, 4, MS>(a, num_sms, st, prep);
-        case 6: return run_tier2<float, 36, 4, MS>(a, num_sms, st, prep);
-        case 7: return run_tier2<float, 40, 4, MS>(a, num_sms, st, prep);
+        case 9: return run_tier2<float, 32, 4, MS>(a, num_sms, st, prep);
+        case 10: return run_tier2<float, 36, 4, MS>(a, num_sms, st, prep);
+        case 11: return run_tier2<float, 40, 4, MS>(a, num_sms, st, prep);
         default: return cudaErrorInvalidValue;
     }
 }
@@ -53,10 +54,11 @@ cudaError_t launch_stream_half(int precision, int ch, const DecodeArgs& a, int s
     return cudaErrorInvalidValue;
 }
 
-cudaError_t launch_decode_tier_half(int precision, int tier, const DecodeArgs& a, int num_sms, cudaStream_t st,
+cudaError_t launch_decode_list_half(int precision, int list, const DecodeArgs& a, int num_sms, cudaStream_t st,
                                     bool prepare_only) {
-    if (precision == 2) return dispatch_half<__half>(tier, a, num_sms, st, prepare_only);
-    if (precision == 3) return dispatch_half<__nv_bfloat16>(tier, a, num_sms, st, prepare_only);
+    if (list < kSmallLists) return launch_decode_small(precision, list, a, num_sms, st, prepare_only);
+    if (precision == 2) return dispatch_half<__half>(list, a, num_sms, st, prepare_only);
+    if (precision == 3) return dispatch_half<__nv_bfloat16>(list, a, num_sms, st, prepare_only);
     return cudaErrorInvalidValue;
 }
 

@@ -128,43 +128,62 @@ __global__ void __launch_bounds__(kCcThreads) sample_cc_kernel(SampleArgs a) {
 
 constexpr int kClsThreads = 256;
 
+// Defect counts and lists.  Bound by latency, not by its bytes (it reads the syndromes once): a
+// block counts its 256 shots per list in shared memory and takes its places with one global
+// atomic per list.  With one global atomic per shot the atomics on a few addresses serialised:
+// 0.66 ms for 10^6 d = 9 code-capacity syndromes, now under 0.02 ms.
 __global__ void __launch_bounds__(kClsThreads) classify_kernel(
     const uint32_t* __restrict__ synd, int64_t shots, int n_words, TierPlan plan,
     int32_t* lists, int32_t* counts, int32_t* max_s, uint8_t* obs_pred, uint8_t* flags,
     int16_t* iters, int32_t* tr_defects, const uint8_t* skip, const uint8_t* skip_obs,
     const int16_t* skip_iters, int64_t list_stride, int32_t item_base) {
+    __shared__ int cnt[kLists], first[kLists], top;
+    const int tid = threadIdx.x;
+    if (tid == 0) top = 0;
     int local_max = 0;
-    for (int64_t shot = (int64_t)blockIdx.x * kClsThreads + threadIdx.x; shot < shots;
-         shot += (int64_t)gridDim.x * kClsThreads) {
-        const uint32_t* w = synd + (size_t)shot * n_words;
-        int s = 0;
-        for (int k = 0; k < n_words; ++k) s += __popc(__ldg(w + k));
-        if (tr_defects) tr_defects[shot] = s;
-        if (skip && skip[shot]) {
-            if (obs_pred) obs_pred[shot] = skip_obs[shot];
-            if (flags) flags[shot] = F_CONVERGED | F_FROM_QBP;
-            if (iters) iters[shot] = skip_iters[shot];
-            continue;
-        }
-        local_max = max(local_max, s);
-        if (s == 0) {
-            if (obs_pred) obs_pred[shot] = 0;
-            if (flags) flags[shot] = F_CONVERGED;
-            if (iters) iters[shot] = 0;
-            continue;
-        }
-        int tier = kGlobalTier;
-        for (int k = 1; k < kGlobalTier; ++k)
-            if (s <= plan.smax[k]) {
-                tier = k;
-                break;
+    for (int64_t base = (int64_t)blockIdx.x * kClsThreads; base < shots; base += (int64_t)gridDim.x * kClsThreads) {
+        if (tid < kLists) cnt[tid] = 0;
+        __syncthreads();
+        const int64_t shot = base + tid;
+        int list = -1, rank = 0;
+        if (shot < shots) {
+            const uint32_t* w = synd + (size_t)shot * n_words;
+            int s = 0;
+            for (int k = 0; k < n_words; ++k) s += __popc(__ldg(w + k));
+            if (tr_defects) tr_defects[shot] = s;
+            if (skip && skip[shot]) {
+                if (obs_pred) obs_pred[shot] = skip_obs[shot];
+                if (flags) flags[shot] = F_CONVERGED | F_FROM_QBP;
+                if (iters) iters[shot] = skip_iters[shot];
+            } else if (s == 0) {
+                if (obs_pred) obs_pred[shot] = 0;
+                if (flags) flags[shot] = F_CONVERGED;
+                if (iters) iters[shot] = 0;
+            } else {
+                local_max = max(local_max, s);
+                list = 0;
+                while (list < kGlobalList && s > plan.smax[list]) ++list;
             }
-        const int pos = atomicAdd(counts + tier, 1);
-        lists[(size_t)tier * list_stride + pos] = item_base | (int32_t)shot;
+        }
+        // rank of the shot among its block's shots of the same list
+        const unsigned peers = __match_any_sync(0xffffffffu, list);
+        const int lane = tid & 31, lead = __ffs((int)peers) - 1;
+        if (list >= 0 && lane == lead) rank = atomicAdd(cnt + list, __popc(peers));
+        rank = __shfl_sync(0xffffffffu, rank, lead) + __popc(peers & ((1u << lane) - 1u));
+        __syncthreads();
+        if (tid < kLists && cnt[tid] > 0) first[tid] = atomicAdd(counts + tid, cnt[tid]);
+        __syncthreads();
+        if (list >= 0) {
+            const int64_t pos = first[list] + rank;
+            lists[(int64_t)list_slot(list) * list_stride + (list_back(list) ? list_stride - 1 - pos : pos)] =
+                item_base | (int32_t)shot;
+        }
+        __syncthreads();
     }
-#pragma unroll
-    for (int off = 16; off; off >>= 1) local_max = max(local_max, __shfl_xor_sync(0xffffffffu, local_max, off));
-    if ((threadIdx.x & 31) == 0 && local_max > 0) atomicMax(max_s, local_max);
+    local_max = __reduce_max_sync(0xffffffffu, local_max);
+    if ((tid & 31) == 0 && local_max > 0) atomicMax(&top, local_max);
+    __syncthreads();
+    if (tid == 0 && top > 0) atomicMax(max_s, top);
 }
 
 constexpr int kCntThreads = 256;

@@ -7,12 +7,12 @@
 
 namespace bp4m {
 
-bool reg_tier_available(int tier) { return tier == 5 || tier == 6; }
+bool reg_list_available(int list) { return list == 9 || list == 10; }
 
-cudaError_t launch_decode_tier_reg(int tier, const DecodeArgs& a, int num_sms, cudaStream_t st, bool prepare_only) {
-    switch (tier) {
-        case 5: return run_reg_tier2<32, 4>(a, num_sms, st, prepare_only);  // 128 rows, 544 threads
-        case 6: return run_reg_tier2<24, 6>(a, num_sms, st, prepare_only);  // 144 rows, 320 threads
+cudaError_t launch_decode_list_reg(int list, const DecodeArgs& a, int num_sms, cudaStream_t st, bool prepare_only) {
+    switch (list) {
+        case 9: return run_reg_tier2<32, 4>(a, num_sms, st, prepare_only);   // 128 rows, 544 threads
+        case 10: return run_reg_tier2<24, 6>(a, num_sms, st, prepare_only);  // 144 rows, 320 threads
         default: return cudaErrorInvalidValue;
     }
 }

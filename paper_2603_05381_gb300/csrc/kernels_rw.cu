@@ -19,10 +19,10 @@ cudaError_t rw_grid(int n_det, int num_sms, int* grid, int64_t* slot_bytes, size
     auto kern = decode_smem_kernel<T, CH, G, false, true>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
+    static std::atomic<int> cache[kOccDevices] = {};
     int per_sm = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, NT, smem);
+    e = resident_blocks(kern, NT, smem, cache, &per_sm);
     if (e != cudaSuccess) return e;
-    if (per_sm < 1) return cudaErrorInvalidConfiguration;
     *grid = per_sm * num_sms;
     *slot_bytes = rw_slot_layout(SMAX, NT, n_det + 1);
     *smem_out = smem;
@@ -44,46 +44,46 @@ cudaError_t run_tier_rw(const DecodeArgs& a, int num_sms, cudaStream_t st, int64
     // every block indexes its own slot: the scratch must hold grid slots of this tier's size
     if (a.gscratch == nullptr || a.rw_slot_bytes != slot || (int64_t)grid * slot > a.gscratch_bytes)
         return cudaErrorInvalidValue;
-    decode_smem_kernel<T, CH, G, false, true><<<grid, CH * G * G, smem, st>>>(a);
+    decode_smem_kernel<T, CH, G, false, true><<<persistent_grid(grid, a), CH * G * G, smem, st>>>(a);
     return cudaGetLastError();
 }
 
-cudaError_t dispatch_rw(int precision, int tier, const DecodeArgs& a, int num_sms, cudaStream_t st,
+cudaError_t dispatch_rw(int precision, int list, const DecodeArgs& a, int num_sms, cudaStream_t st,
                         int64_t* query) {
     if (precision == 0) {
-        switch (tier) {
-            case 1: return run_tier_rw<double, 16, 2>(a, num_sms, st, query);
-            case 2: return run_tier_rw<double, 16, 4>(a, num_sms, st, query);
-            case 3: return run_tier_rw<double, 28, 4>(a, num_sms, st, query);
+        switch (list) {
+            case 3: return run_tier_rw<double, 16, 2>(a, num_sms, st, query);
+            case 5: return run_tier_rw<double, 16, 4>(a, num_sms, st, query);
+            case 8: return run_tier_rw<double, 28, 4>(a, num_sms, st, query);
             default: return cudaErrorInvalidValue;
         }
     }
-    switch (tier) {
-        case 1: return run_tier_rw<float, 32, 1>(a, num_sms, st, query);
-        case 2: return run_tier_rw<float, 32, 2>(a, num_sms, st, query);
-        case 3: return run_tier_rw<float, 24, 4>(a, num_sms, st, query);
-        case 4: return run_tier_rw<float, 28, 4>(a, num_sms, st, query);
-        case 5: return run_tier_rw<float, 32, 4>(a, num_sms, st, query);
-        case 6: return run_tier_rw<float, 36, 4>(a, num_sms, st, query);
-        case 7: return run_tier_rw<float, 40, 4>(a, num_sms, st, query);
+    switch (list) {
+        case 3: return run_tier_rw<float, 32, 1>(a, num_sms, st, query);
+        case 5: return run_tier_rw<float, 32, 2>(a, num_sms, st, query);
+        case 7: return run_tier_rw<float, 24, 4>(a, num_sms, st, query);
+        case 8: return run_tier_rw<float, 28, 4>(a, num_sms, st, query);
+        case 9: return run_tier_rw<float, 32, 4>(a, num_sms, st, query);
+        case 10: return run_tier_rw<float, 36, 4>(a, num_sms, st, query);
+        case 11: return run_tier_rw<float, 40, 4>(a, num_sms, st, query);
         default: return cudaErrorInvalidValue;
     }
 }
 
 }  // namespace
 
-size_t rw_scratch_bytes(int precision, int tier, int n_det, int num_sms, int64_t* slot_bytes) {
+size_t rw_scratch_bytes(int precision, int list, int n_det, int num_sms, int64_t* slot_bytes) {
     DecodeArgs a;
     a.tb.n_det = n_det;
     int64_t q[2] = {0, 0};
-    if (dispatch_rw(precision, tier, a, num_sms, 0, q) != cudaSuccess) return 0;
+    if (dispatch_rw(precision, list, a, num_sms, 0, q) != cudaSuccess) return 0;
     if (slot_bytes) *slot_bytes = q[1];
     return (size_t)q[0];
 }
 
-cudaError_t launch_decode_tier_rw(int precision, int tier, const DecodeArgs& a, int num_sms,
+cudaError_t launch_decode_list_rw(int precision, int list, const DecodeArgs& a, int num_sms,
                                   cudaStream_t st) {
-    return dispatch_rw(precision, tier, a, num_sms, st, nullptr);
+    return dispatch_rw(precision, list, a, num_sms, st, nullptr);
 }
 
 }  // namespace bp4m
