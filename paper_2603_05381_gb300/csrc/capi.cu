@@ -588,7 +588,7 @@ int decode_device(bp4m_graph* g, Workspace& w, int ty, const uint32_t* synd, int
         int64_t slot[kLists] = {};
         for (int c = 0; c < kGlobalList; ++c) {
             if (!plan.used(c)) continue;
-            const size_t b = rw_scratch_bytes(prec, c, g->host.t[ty].n_det, g->num_sms, &slot[c]);
+            const size_t b = rw_scratch_bytes(prec, c, g->host.t[ty].n_det, g->host.n_units, g->num_sms, &slot[c]);
             if (b == 0) return fail(BP4M_ECUDA, "B-BP4MF: no launch configuration for a reweighting tier");
             need = std::max(need, b);
         }

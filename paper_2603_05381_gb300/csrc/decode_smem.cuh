@@ -377,9 +377,9 @@ __global__ void __launch_bounds__(block_threads(CH, G, (int)sizeof(T), (int)size
                                 : nullptr;
     double* Wsh = reinterpret_cast<double*>(rw_slot);
     double* rw_dist = Wsh + SMAX * SMAX;
-    unsigned char* Psh = reinterpret_cast<unsigned char*>(rw_dist + (NT / 32) * rw_nodes);
-    unsigned char* rw_done = Psh + SMAX * SMAX;
-    unsigned char* rw_par = rw_done + (NT / 32) * rw_nodes;
+    double* rw_w = rw_dist + (NT / 32) * rw_nodes;  // [rw_units] weights of the shot's qubits
+    uint32_t* rw_pred = reinterpret_cast<uint32_t*>(rw_w + a.rw_units);
+    unsigned char* Psh = reinterpret_cast<unsigned char*>(rw_pred + (NT / 32) * rw_nodes);
     __shared__ int sh_item, sh_s, sh_flags, sh_best_par, sh_best_forced, sh_improve, sh_use_best;
     __shared__ double sh_best_w;
     __shared__ int sh_next_code[2], sh_next_s[2];  // HELP: the shots fetched ahead
@@ -555,83 +555,104 @@ __global__ void __launch_bounds__(block_threads(CH, G, (int)sizeof(T), (int)size
                 }
             }
         } else {
-            // Dijkstra from every defect (one warp per source): nodes popped in (distance,
-            // index) order, predecessor changed only on a strict improvement, the boundary
-            // node n a sink; edge weight |ln((1-P)/P)| of the qubit behind the edge (edges
-            // above one half were flipped out of the syndrome), floored at kRwMinWeight
-            double* dist = rw_dist + warp * rw_nodes;
-            unsigned char* done = rw_done + warp * rw_nodes;
-            unsigned char* par = rw_par + warp * rw_nodes;
-            const double* post = a.rw_post + (size_t)shot * a.rw_units;
-            const double dinf = Num<double>::pinf();
+            // Shortest paths from every defect (one warp per source) over edge weights
+            // |ln((1-P)/P)| of the qubit behind the edge (edges above one half were flipped out of
+            // the syndrome), floored at kRwMinWeight; the boundary node n is a sink.  Distances and
+            // parities are those of Dijkstra's algorithm that pops nodes in (distance, index) order
+            // and changes a predecessor only on a strict improvement: rounding is monotone and
+            // weights are positive, so relaxing every node from its neighbours until nothing
+            // changes ends in the same distances, and v's predecessor is the neighbour u, first in
+            // (distance, index) order, then the first entry of v's list, with dist[u] + w equal to
+            // dist[v].  Weights are taken once per qubit of the shot: a logarithm per relaxed edge
+            // and source, by one lane, was most of this stage (FP64 runs at two operations a clock
+            // and SM): 28.5 -> 3.2 ms for 10,000 d = 9 shots of both stages.  Distances are positive, so
+            // they compare as integers.
+            for (int u = tid; u < a.rw_units; u += NT) {
+                double pq = a.rw_post[(size_t)shot * a.rw_units + u];
+                pq = pq < 1e-300 ? 1e-300 : (pq > 1.0 - 1e-16 ? 1.0 - 1e-16 : pq);
+                // an edge above one half was taken as present (flipped out of the syndrome): it
+                // weighs as its complement
+                if (pq > 0.5) pq = 1.0 - pq;
+                rw_w[u] = fmax(log((1.0 - pq) / pq), kRwMinWeight);
+            }
+            __syncthreads();
+            long long* const dist = reinterpret_cast<long long*>(rw_dist + warp * rw_nodes);
+            uint32_t* const pred = rw_pred + warp * rw_nodes;
+            const long long dinf = __double_as_longlong(Num<double>::pinf());
             for (int r = warp; r < s; r += NT / 32) {
-                for (int v = lane; v < rw_nodes; v += 32) {
-                    dist[v] = dinf;
-                    done[v] = 0;
-                    par[v] = 0;
-                }
+                const int src = dets[r];
+                for (int v = lane; v < rw_nodes; v += 32) dist[v] = v == src ? 0 : dinf;
                 __syncwarp();
-                if (lane == 0) dist[dets[r]] = 0.0;
-                __syncwarp();
-                for (int step = 0; step < rw_nodes; ++step) {
-                    double bd = dinf;
-                    int bi = 0x7fffffff;
-                    for (int v = lane; v < rw_nodes; v += 32)
-                        if (!done[v] && dist[v] < bd) {
-                            bd = dist[v];
-                            bi = v;
-                        }
-#pragma unroll
-                    for (int off = 16; off; off >>= 1) {
-                        const double od = __shfl_xor_sync(kFull, bd, off);
-                        const int oi = __shfl_xor_sync(kFull, bi, off);
-                        if (od < bd || (od == bd && oi < bi)) {
-                            bd = od;
-                            bi = oi;
-                        }
-                    }
-                    if (bd == dinf) break;
-                    if (lane == 0) {
-                        done[bi] = 1;
-                        if (bi != n) {
-                            for (int e = a.rw_off[bi]; e < a.rw_off[bi + 1]; ++e) {
+                bool again = true;
+                for (int sweep = 0; again && sweep <= rw_nodes; ++sweep) {  // (a path has fewer edges than nodes)
+                    bool changed = false;
+                    for (int v0 = 0; v0 < n; v0 += 32) {
+                        const int v = v0 + lane;
+                        long long best = v < n ? dist[v] : 0;
+                        bool up = false;
+                        if (v < n) {
+                            const int e1 = a.rw_off[v + 1];
+                            for (int e = a.rw_off[v]; e < e1; ++e) {
                                 const uint32_t pk = a.rw_adj[e];
-                                const int v = (int)(pk & 0x7FFFu);
-                                double pq = post[(pk >> 15) & 0x7FFFu];
-                                pq = pq < 1e-300 ? 1e-300 : (pq > 1.0 - 1e-16 ? 1.0 - 1e-16 : pq);
-                                // an edge above one half was taken as present (flipped out of
-                                // the syndrome): it weighs as its complement
-                                if (pq > 0.5) pq = 1.0 - pq;
-                                const double nd = bd + fmax(log((1.0 - pq) / pq), kRwMinWeight);
-                                if (nd < dist[v]) {
-                                    dist[v] = nd;
-                                    par[v] = par[bi] ^ (unsigned char)(pk >> 31);
+                                const int u = (int)(pk & 0x7FFFu);
+                                if (u == n) continue;
+                                const long long nd = __double_as_longlong(__longlong_as_double(dist[u]) + rw_w[(pk >> 15) & 0x7FFFu]);
+                                if (nd < best) {
+                                    best = nd;
+                                    up = true;
                                 }
                             }
                         }
+                        __syncwarp();
+                        if (up) dist[v] = best;
+                        changed |= up;
+                        __syncwarp();
                     }
-                    __syncwarp();
+                    again = __any_sync(kFull, changed);
                 }
+                // the boundary's distance, and every node's predecessor (node | obs << 15)
+                for (int v = lane; v < rw_nodes; v += 32) {
+                    const int e1 = a.rw_off[v + 1];
+                    long long best = v == n ? dinf : dist[v], du = dinf;
+                    uint32_t p = 0xFFFFFFFFu;
+                    for (int e = a.rw_off[v]; e < e1; ++e) {
+                        const uint32_t pk = a.rw_adj[e];
+                        const int u = (int)(pk & 0x7FFFu);
+                        if (u == n) continue;
+                        const long long d = dist[u];
+                        const long long nd = __double_as_longlong(__longlong_as_double(d) + rw_w[(pk >> 15) & 0x7FFFu]);
+                        const bool better = v == n && nd < best;
+                        if (nd != dinf && (better || (nd == best && d < du))) {
+                            best = nd;
+                            du = d;
+                            p = (uint32_t)u | (pk >> 31) << 15;
+                        }
+                    }
+                    pred[v] = v == src ? 0xFFFFFFFFu : p;
+                    if (v == n) dist[n] = best;
+                }
+                __syncwarp();
                 for (int k = r + lane; k < s; k += 32) {
                     const int tgt = k == r ? n : dets[k];
-                    Wsh[r * SMAX + k] = dist[tgt];
-                    Psh[r * SMAX + k] = par[tgt];
+                    unsigned char par = 0;
+                    for (uint32_t p = pred[tgt]; p != 0xFFFFFFFFu; p = pred[p & 0x7FFFu]) par ^= (unsigned char)(p >> 15);
+                    Wsh[r * SMAX + k] = __longlong_as_double(dist[tgt]);
+                    Psh[r * SMAX + k] = par;
                 }
                 __syncwarp();
             }
             __syncthreads();
+            // priors of the pairs k >= r, mirrored
             for (int r = warp; r < s; r += NT / 32) {
                 for (int k = lane; k < SMAX; k += 32) {
-                    if (k < s) {
-                        if (k < r) {
-                            Wsh[r * SMAX + k] = Wsh[k * SMAX + r];
-                            Psh[r * SMAX + k] = Psh[k * SMAX + r];
-                        }
-                        const double W = k < r ? Wsh[k * SMAX + r] : Wsh[r * SMAX + k];
-                        const double l = W == dinf ? -1.0e30 : -W - log1p(-exp(-W));
-                        Lm[r * P + k] = (T)(l * kLog2e);
-                    } else {
+                    if (k >= s) {
                         Lm[r * P + k] = ninf;
+                    } else if (k >= r) {
+                        const double W = Wsh[r * SMAX + k];
+                        const double l = W == Num<double>::pinf() ? -1.0e30 : -W - log1p(-exp(-W));
+                        Lm[r * P + k] = Lm[k * P + r] = (T)(l * kLog2e);
+                        Wsh[k * SMAX + r] = W;
+                        Psh[k * SMAX + r] = Psh[r * SMAX + k];
                     }
                     Mt[r * PM + k] = MS(0.f);
                 }
@@ -1248,11 +1269,11 @@ constexpr int kRows32[kGlobalList] = {8, 16, 24, 32, 48, 64, 80, 96, 112, 128, 1
 constexpr int kRowsRw32[kGlobalList] = {0, 0, 0, 32, 0, 64, 0, 96, 112, 128, 144, 160};
 constexpr int kRows64[kGlobalList] = {0, 0, 0, 32, 0, 64, 0, 0, 112, 0, 0, 0};
 
-// Bytes of one RW scratch slot: W [SMAX][SMAX] doubles, Dijkstra distances [warps][nodes]
-// doubles, parity [SMAX][SMAX] bytes, done and parity flags [warps][nodes] bytes.
-inline int64_t rw_slot_layout(int smax, int nt, int nodes) {
-    const int64_t b = 8 * ((int64_t)smax * smax + (int64_t)(nt / 32) * nodes) + (int64_t)smax * smax +
-                      2 * (int64_t)(nt / 32) * nodes;
+// Bytes of one RW scratch slot: W [SMAX][SMAX] doubles, path distances [warps][nodes] doubles,
+// qubit weights [units] doubles, predecessors [warps][nodes] words, parity [SMAX][SMAX] bytes.
+inline int64_t rw_slot_layout(int smax, int nt, int nodes, int units) {
+    const int64_t b = 8 * ((int64_t)smax * smax + (int64_t)(nt / 32) * nodes + units) +
+                      4 * (int64_t)(nt / 32) * nodes + (int64_t)smax * smax;
     return (b + 255) / 256 * 256;
 }
 

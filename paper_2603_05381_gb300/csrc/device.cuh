@@ -249,7 +249,7 @@ cudaError_t launch_decode_list(int precision, int list, const DecodeArgs& a, int
 // uses.  rw_scratch_bytes() is the global scratch the launch of a list needs for a graph
 // of n_det detectors (one slot per resident block) and sets *slot_bytes; the caller
 // passes that scratch in a.gscratch and the slot size in a.rw_slot_bytes.
-size_t rw_scratch_bytes(int precision, int list, int n_det, int num_sms, int64_t* slot_bytes);
+size_t rw_scratch_bytes(int precision, int list, int n_det, int units, int num_sms, int64_t* slot_bytes);
 cudaError_t launch_decode_list_rw(int precision, int list, const DecodeArgs& a, int num_sms,
                                   cudaStream_t st);
 // Smallest edge weight of the reweighted graph: posteriors at or above one half would give

@@ -27,19 +27,23 @@ __device__ __forceinline__ int anti(bool xcheck, int E) {
     return xcheck ? (E == 2 || E == 3) : (E == 1 || E == 2);
 }
 
+// ln(e^a + e^b); the larger term's exponential is exactly 1.
 template <typename T>
 __device__ __forceinline__ T lse2(T a, T b) {
-    const T m = a > b ? a : b;
+    const bool ab = a > b;
+    const T m = ab ? a : b, lo = ab ? b : a;
     if (m == -INFINITY) return m;
-    return m + log(exp(a - m) + exp(b - m));
+    return m + log(exp(lo - m) + T(1));
 }
 
 template <typename T>
 __global__ void __launch_bounds__(kQbpThreads) qbp_kernel(QbpArgs a) {
     extern __shared__ __align__(16) unsigned char smem[];
     const int nc = a.n_checks, n = a.n_qubits;
-    T* mu = reinterpret_cast<T*>(smem);             // [nc][4]
-    T* dl = mu + 4 * nc;                            // [nc][4]
+    // [nc][4]: tanh(mu_vc / 2), taken once per edge where it is made (its check's other edges each
+    // read it)
+    T* th = reinterpret_cast<T*>(smem);
+    T* dl = th + 4 * nc;                            // [nc][4]
     unsigned char* zc = reinterpret_cast<unsigned char*>(dl + 4 * nc);  // [nc]
     unsigned char* dec = zc + nc;                   // [n]
     const T p = (T)a.p;
@@ -78,7 +82,7 @@ __global__ void __launch_bounds__(kQbpThreads) qbp_kernel(QbpArgs a) {
                 // commuting: I and (X for an X-check, Z for a Z-check); anticommuting: the rest
                 const T num = lse2(lq[0], xc ? lq[1] : lq[3]);
                 const T den = lse2(lq[2], xc ? lq[3] : lq[1]);
-                mu[e] = num - den;
+                th[e] = tanh((num - den) * T(0.5));
             }
             __syncthreads();
             // check -> qubit
@@ -87,7 +91,7 @@ __global__ void __launch_bounds__(kQbpThreads) qbp_kernel(QbpArgs a) {
                 if (a.chk_q[e] < 0) continue;
                 T prod = T(1);
                 for (int j = 0; j < 4; ++j)
-                    if (j != j0 && a.chk_q[c * 4 + j] >= 0) prod *= tanh(mu[c * 4 + j] * T(0.5));
+                    if (j != j0 && a.chk_q[c * 4 + j] >= 0) prod *= th[c * 4 + j];
                 prod = prod > T(1) - clampv ? T(1) - clampv : (prod < clampv - T(1) ? clampv - T(1) : prod);
                 dl[e] = (zc[c] ? T(-2) : T(2)) * atanh(prod);
             }

@@ -1,8 +1,8 @@
 // Second stage of B-BP4MF (Sec. "Belief-BP4MF (B-BP4MF)", Sec. "Correlated decoding"):
-// the shared-memory decoding kernel in its reweighting mode.  Each block first runs
-// Dijkstra from every unsatisfied check of its shot over the decoding graph whose edge
-// weights come from the first stage's qubit posteriors, then BP4MF on the resulting
-// priors.  Per-shot W, parity and the Dijkstra state live in a global scratch slot per
+// the shared-memory decoding kernel in its reweighting mode.  Each block first finds the
+// shortest paths from every unsatisfied check of its shot over the decoding graph whose edge
+// weights come from the first stage's qubit posteriors, then runs BP4MF on the resulting
+// priors.  Per-shot W, parity and the path state live in a global scratch slot per
 // resident block.
 #include <cuda_runtime.h>
 
@@ -13,7 +13,7 @@ namespace bp4m {
 namespace {
 
 template <typename T, int CH, int G>
-cudaError_t rw_grid(int n_det, int num_sms, int* grid, int64_t* slot_bytes, size_t* smem_out) {
+cudaError_t rw_grid(int n_det, int units, int num_sms, int* grid, int64_t* slot_bytes, size_t* smem_out) {
     constexpr int SMAX = CH * G, NT = CH * G * G;
     const size_t smem = smem_bytes_of<T, CH, G, T, true>();
     auto kern = decode_smem_kernel<T, CH, G, false, true>;
@@ -24,7 +24,7 @@ cudaError_t rw_grid(int n_det, int num_sms, int* grid, int64_t* slot_bytes, size
     e = resident_blocks(kern, NT, smem, cache, &per_sm);
     if (e != cudaSuccess) return e;
     *grid = per_sm * num_sms;
-    *slot_bytes = rw_slot_layout(SMAX, NT, n_det + 1);
+    *slot_bytes = rw_slot_layout(SMAX, NT, n_det + 1, units);
     *smem_out = smem;
     return cudaSuccess;
 }
@@ -34,7 +34,7 @@ cudaError_t run_tier_rw(const DecodeArgs& a, int num_sms, cudaStream_t st, int64
     int grid = 0;
     int64_t slot = 0;
     size_t smem = 0;
-    cudaError_t e = rw_grid<T, CH, G>(a.tb.n_det, num_sms, &grid, &slot, &smem);
+    cudaError_t e = rw_grid<T, CH, G>(a.tb.n_det, a.rw_units, num_sms, &grid, &slot, &smem);
     if (e != cudaSuccess) return e;
     if (query) {
         query[0] = (int64_t)grid * slot;
@@ -72,9 +72,10 @@ cudaError_t dispatch_rw(int precision, int list, const DecodeArgs& a, int num_sm
 
 }  // namespace
 
-size_t rw_scratch_bytes(int precision, int list, int n_det, int num_sms, int64_t* slot_bytes) {
+size_t rw_scratch_bytes(int precision, int list, int n_det, int units, int num_sms, int64_t* slot_bytes) {
     DecodeArgs a;
     a.tb.n_det = n_det;
+    a.rw_units = units;
     int64_t q[2] = {0, 0};
     if (dispatch_rw(precision, list, a, num_sms, 0, q) != cudaSuccess) return 0;
     if (slot_bytes) *slot_bytes = q[1];
