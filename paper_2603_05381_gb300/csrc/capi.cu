@@ -95,6 +95,10 @@ struct Workspace {
     cudaStream_t aux = nullptr;   // second stream: classes of few shots run beside the others
     cudaEvent_t ev_sub = nullptr, ev_fork = nullptr, ev_join = nullptr;
     cudaEvent_t ev_small = nullptr;
+    // staging of small host batches (decode_host): one device block and its pinned mirror
+    unsigned char* hb_dev = nullptr;
+    unsigned char* hb_pin = nullptr;
+    size_t hb_bytes = 0;
     // B-BP4MF first stage
     int64_t qcap = 0;
     uint8_t* qconv = nullptr;
@@ -349,6 +353,8 @@ void free_ws(Workspace& w) {
     cudaFreeHost(w.host_small);
     cudaFreeHost(w.host_ctr);
     if (w.ev_small) cudaEventDestroy(w.ev_small);
+    cudaFree(w.hb_dev);
+    cudaFreeHost(w.hb_pin);
     cudaFree(w.qconv);
     cudaFree(w.qobs);
     cudaFree(w.qiters);
@@ -397,7 +403,17 @@ int ensure_gscratch(Workspace& w, size_t bytes) {
     return BP4M_OK;
 }
 
+// The second stream of the global tier and the events that fork and join it.
+int ensure_aux(Workspace& w) {
+    if (!w.aux) CK(cudaStreamCreateWithFlags(&w.aux, cudaStreamNonBlocking));
+    if (!w.ev_fork) CK(cudaEventCreateWithFlags(&w.ev_fork, cudaEventDisableTiming));
+    if (!w.ev_join) CK(cudaEventCreateWithFlags(&w.ev_join, cudaEventDisableTiming));
+    return BP4M_OK;
+}
+
 int ensure_split(Workspace& w, int64_t cap) {
+    const int rc = ensure_aux(w);
+    if (rc) return rc;
     if (w.sub_cap >= cap) return BP4M_OK;
     cudaFree(w.sub);
     cudaFree(w.subctr);
@@ -408,10 +424,7 @@ int ensure_split(Workspace& w, int64_t cap) {
     CK(dalloc(&w.subctr, 2 * kMaxGlobalClasses));
     w.sub_cap = cap;
     if (!w.host_sub) CK(cudaMallocHost(reinterpret_cast<void**>(&w.host_sub), kMaxGlobalClasses * sizeof(int32_t)));
-    if (!w.aux) CK(cudaStreamCreateWithFlags(&w.aux, cudaStreamNonBlocking));
     if (!w.ev_sub) CK(cudaEventCreateWithFlags(&w.ev_sub, cudaEventDisableTiming));
-    if (!w.ev_fork) CK(cudaEventCreateWithFlags(&w.ev_fork, cudaEventDisableTiming));
-    if (!w.ev_join) CK(cudaEventCreateWithFlags(&w.ev_join, cudaEventDisableTiming));
     return BP4M_OK;
 }
 
@@ -528,6 +541,61 @@ struct Stage2 {
     const double* post = nullptr;       // [shots][n_units] posteriors of this type
 };
 
+// Launch arguments common to every list of a batch.
+DecodeArgs decode_args(const bp4m_graph* g, int ty, const uint32_t* synd, int64_t shots, int T, const bp4m_opts* o,
+                       uint8_t* obs_pred, uint8_t* flags, int16_t* iters, unsigned long long* ctr) {
+    DecodeArgs a;
+    a.tb = dev_tables(g, ty);
+    a.synd = synd;
+    a.shots = shots;
+    a.T = T;
+    a.early_exit = o->early_exit ? 1 : 0;
+    a.decoder = o->decoder;
+    a.forced_static = o->forced == BP4M_FORCED_STATIC ? 1 : 0;
+    a.stream_cl = o->stream_cluster;
+    a.tile_form = o->tile_form;
+    a.alpha = o->alpha;
+    a.obs_pred = obs_pred;
+    a.flags = flags;
+    a.iters = iters;
+    a.ctr = ctr;
+    return a;
+}
+
+// Launches the width classes of the global tier whose counts the host knows (class c: host_cnt[c]
+// items at lists[c], device count and work counter at counts[c] and nexts[c]).  A class of fewer
+// shots than half its resident blocks (typically a few shots above the bulk's width) runs on the
+// second stream beside the others with its own scratch, instead of holding the stream for a
+// whole shot's decode on a few SMs; empty classes are skipped.
+int launch_global_counted(Workspace& w, const DecodeArgs& a, const GlobalPlan& p, int pio, const bp4m_opts* o,
+                          const int32_t* host_cnt, const int32_t* const* lists, const int32_t* counts, int32_t* nexts,
+                          cudaStream_t st) {
+    const size_t esz = pio == 0 ? sizeof(double) : sizeof(float);
+    CK(cudaEventRecord(w.ev_fork, st));
+    CK(cudaStreamWaitEvent(w.aux, w.ev_fork, 0));
+    // small classes first, so that their few blocks hold their SMs before the large
+    // classes' persistent blocks fill the rest
+    for (int pass = 0; pass < 2; ++pass)
+        for (int c = 0; c < p.gc.n; ++c) {
+            const int cnt = host_cnt[c];
+            const bool small = 2 * cnt < p.full[c];
+            if (cnt <= 0 || small != (pass == 0)) continue;
+            DecodeArgs b = a;
+            b.list = lists[c];
+            b.list_dir = 1;
+            b.count = counts + c;
+            b.next = nexts + c;
+            b.gslot_elems = (int64_t)(p.slot_bytes[c] / esz / 3);
+            b.gsmax = p.gsmax[c];
+            b.stream_cl = stream_cluster_for(pio, b.gsmax, o->stream_cluster, cnt, p.full[c]);
+            if (small) b.gscratch = static_cast<unsigned char*>(w.gscratch) + p.need;
+            CK(launch_decode_global(pio, b, small ? cnt : std::min(cnt, p.full[c]), small ? w.aux : st));
+        }
+    CK(cudaEventRecord(w.ev_join, w.aux));
+    CK(cudaStreamWaitEvent(st, w.ev_join, 0));
+    return BP4M_OK;
+}
+
 int decode_device(bp4m_graph* g, Workspace& w, int ty, const uint32_t* synd, int64_t shots, int T,
                   const bp4m_opts* o, uint8_t* obs_pred, uint8_t* flags, int16_t* iters,
                   const bp4m_trace* tr, cudaStream_t st, const Stage2* rw = nullptr) {
@@ -554,21 +622,7 @@ int decode_device(bp4m_graph* g, Workspace& w, int ty, const uint32_t* synd, int
                        cudaMemcpyDeviceToHost, st));
     CK(cudaEventRecord(w.ev_small, st));
     CK(cudaEventSynchronize(w.ev_small));
-    DecodeArgs a;
-    a.tb = dev_tables(g, ty);
-    a.synd = synd;
-    a.shots = shots;
-    a.T = T;
-    a.early_exit = o->early_exit ? 1 : 0;
-    a.decoder = o->decoder;
-    a.forced_static = o->forced == BP4M_FORCED_STATIC ? 1 : 0;
-    a.stream_cl = o->stream_cluster;
-    a.tile_form = o->tile_form;
-    a.alpha = o->alpha;
-    a.obs_pred = obs_pred;
-    a.flags = flags;
-    a.iters = iters;
-    a.ctr = w.ctr;
+    DecodeArgs a = decode_args(g, ty, synd, shots, T, o, obs_pred, flags, iters, w.ctr);
     if (tr) {
         a.tr_lambda = tr->lambda;
         a.tr_partner = tr->partner;
@@ -641,40 +695,199 @@ int decode_device(bp4m_graph* g, Workspace& w, int ty, const uint32_t* synd, int
                                        g->num_sms, st);
             if (rc) return rc;
         } else {
-            // partition, then read the class counts: a class of fewer shots than half its
-            // resident blocks (typically a few shots above the bulk's width) runs on the
-            // second stream beside the others with its own scratch, instead of holding the
-            // stream for a whole shot's decode on a few SMs; empty classes are skipped
-            const size_t esz = prec == 0 ? sizeof(double) : sizeof(float);
+            // partition, then read the class counts
             CK(cudaMemsetAsync(w.subctr, 0, 2 * kMaxGlobalClasses * sizeof(int32_t), st));
             CK(launch_partition_global(a, p.gc, w.sub, shots, w.subctr, n_glob, g->num_sms, st));
             CK(cudaMemcpyAsync(w.host_sub, w.subctr, p.gc.n * sizeof(int32_t), cudaMemcpyDeviceToHost, st));
             CK(cudaEventRecord(w.ev_sub, st));
             CK(cudaEventSynchronize(w.ev_sub));
-            CK(cudaEventRecord(w.ev_fork, st));
-            CK(cudaStreamWaitEvent(w.aux, w.ev_fork, 0));
-            // small classes first, so that their few blocks hold their SMs before the large
-            // classes' persistent blocks fill the rest
-            for (int pass = 0; pass < 2; ++pass)
-                for (int c = 0; c < p.gc.n; ++c) {
-                    const int cnt = w.host_sub[c];
-                    const bool small = 2 * cnt < p.full[c];
-                    if (cnt <= 0 || small != (pass == 0)) continue;
-                    DecodeArgs b = a;
-                    b.list = w.sub + (size_t)c * shots;
-                    b.count = w.subctr + c;
-                    b.next = w.subctr + kMaxGlobalClasses + c;
-                    b.gslot_elems = (int64_t)(p.slot_bytes[c] / esz / 3);
-                    b.gsmax = p.gsmax[c];
-                    b.stream_cl = stream_cluster_for(pio, b.gsmax, o->stream_cluster, cnt, p.full[c]);
-                    if (small) b.gscratch = static_cast<unsigned char*>(w.gscratch) + p.need;
-                    CK(launch_decode_global(pio, b, small ? cnt : std::min(cnt, p.full[c]), small ? w.aux : st));
-                }
-            CK(cudaEventRecord(w.ev_join, w.aux));
-            CK(cudaStreamWaitEvent(st, w.ev_join, 0));
+            const int32_t* lists[kMaxGlobalClasses];
+            for (int c = 0; c < p.gc.n; ++c) lists[c] = w.sub + (size_t)c * shots;
+            rc = launch_global_counted(w, a, p, pio, o, w.host_sub, lists, w.subctr, w.subctr + kMaxGlobalClasses, st);
+            if (rc) return rc;
         }
         ps.end();
     }
+    return BP4M_OK;
+}
+
+// Small host batches.  Latency bounds these: of a one-shot d = 5 request's 114 us, the decoding is
+// about 10; the rest went into launches for empty lists, a wait for the counts, and a pageable
+// copy per buffer.  The host counts the defects while it stages the syndromes in pinned memory, so
+// that one copy brings syndromes, lists and zeroed counters, only the lists in use are launched,
+// and one copy takes all results back.  Larger batches are counted on the device: the count of
+// kHostBatch shots costs the host tens of microseconds.  Measured: one d = 5 shot 93 -> 45 us, seven
+// d = 19 shots (one launch for their width classes, below) 875 -> 408 us.
+constexpr int64_t kHostBatch = 2048;
+
+// One block on both sides: obs, flags, iters and the counters come back; the counters, the lists'
+// counts and work counters, the items and the syndromes go up.
+struct HostBatch {
+    size_t flags, iters, ctr, cnt, items, synd, sdef, bytes;  // sdef (defect counts): host side only
+    HostBatch(int64_t n, int nw) {
+        flags = (size_t)n;
+        iters = (2 * (size_t)n + 1) / 2 * 2;
+        ctr = (iters + 2 * (size_t)n + 7) / 8 * 8;
+        cnt = ctr + C_NUM * sizeof(unsigned long long);
+        items = cnt + kInts * sizeof(int32_t);
+        synd = items + (size_t)n * sizeof(int32_t);
+        sdef = synd + (size_t)n * nw * sizeof(uint32_t);
+        bytes = sdef + (size_t)n * sizeof(uint16_t);
+    }
+    // counts and work counters of the lists, then of the global tier's width classes
+    static constexpr int kInts = 2 * kLists + 2 * kMaxGlobalClasses;
+};
+
+int decode_host(bp4m_graph* g, Workspace& w, int ty, const uint32_t* synd, int64_t shots, int T, const bp4m_opts* o,
+                uint8_t* obs_pred, uint8_t* converged, int16_t* iters_used, cudaStream_t st) {
+    const int pio = o->precision == BP4M_FP64 ? 0 : o->precision == BP4M_FP32 ? 1 : o->precision;
+    if (!g->prepared[pio]) {
+        CK(prepare_decode_kernels(pio));
+        g->prepared[pio] = true;
+    }
+    const int nw = n_words_of(g, ty);
+    const HostBatch L(shots, nw);
+    if (w.hb_bytes < L.bytes) {
+        // grown to the next power of two, so that requests of many sizes reallocate rarely
+        size_t b = 4096;
+        while (b < L.bytes) b *= 2;
+        cudaFree(w.hb_dev);
+        cudaFreeHost(w.hb_pin);
+        w.hb_dev = w.hb_pin = nullptr;
+        w.hb_bytes = 0;
+        CK(cudaMalloc(reinterpret_cast<void**>(&w.hb_dev), b));
+        CK(cudaMallocHost(reinterpret_cast<void**>(&w.hb_pin), b));
+        w.hb_bytes = b;
+    }
+    unsigned char* const hp = w.hb_pin;
+    unsigned char* const dp = w.hb_dev;
+    std::memset(hp + L.ctr, 0, L.items - L.ctr);
+    std::memcpy(hp + L.synd, synd, (size_t)shots * nw * sizeof(uint32_t));
+    // defect counts, lists by counting
+    const TierPlan plan = tier_plan(pio == 0 ? 0 : 1);
+    uint16_t* const sdef = reinterpret_cast<uint16_t*>(hp + L.sdef);
+    int max_s = 0;
+    int32_t* const cnt = reinterpret_cast<int32_t*>(hp + L.cnt);
+    int32_t* const gcnt = cnt + 2 * kLists;
+    for (int64_t k = 0; k < shots; ++k) {
+        const uint32_t* row = synd + (size_t)k * nw;
+        int s = 0;
+        for (int q = 0; q < nw; ++q) s += __builtin_popcount(row[q]);
+        sdef[k] = (uint16_t)s;
+        max_s = std::max(max_s, s);
+    }
+    auto list_of = [&](int s) {
+        int c = 0;
+        while (c < kGlobalList && s > plan.smax[c]) ++c;
+        return c;
+    };
+    const bool glob = list_of(max_s) == kGlobalList;
+    GlobalPlan p;
+    if (glob) p = global_plan(pio, max_s, g->num_sms);
+    auto class_of = [&](int s) {
+        int c = 0;
+        while (c + 1 < p.gc.n && s > p.gc.smax[c]) ++c;
+        return c;
+    };
+    for (int64_t k = 0; k < shots; ++k) {
+        if (sdef[k] == 0) continue;
+        const int c = list_of(sdef[k]);
+        if (c == kGlobalList)
+            ++gcnt[class_of(sdef[k])];
+        else
+            ++cnt[c];
+    }
+    int32_t first[kLists], gfirst[kMaxGlobalClasses], pos = 0;
+    for (int c = 0; c < kGlobalList; ++c) {
+        first[c] = pos;
+        pos += cnt[c];
+    }
+    for (int c = 0; c < kMaxGlobalClasses; ++c) {
+        gfirst[c] = pos;
+        pos += gcnt[c];
+    }
+    int32_t* const items = reinterpret_cast<int32_t*>(hp + L.items);
+    {
+        int32_t at[kLists], gat[kMaxGlobalClasses];
+        std::copy(first, first + kLists, at);
+        std::copy(gfirst, gfirst + kMaxGlobalClasses, gat);
+        for (int64_t k = 0; k < shots; ++k) {
+            if (sdef[k] == 0) continue;
+            const int c = list_of(sdef[k]);
+            items[c == kGlobalList ? gat[class_of(sdef[k])]++ : at[c]++] = (int32_t)k;
+        }
+    }
+    if (glob) {
+        int rc = ensure_gscratch(w, p.need + (p.gc.n > 1 ? p.need_small : 0));
+        if (rc) return rc;
+        rc = ensure_aux(w);
+        if (rc) return rc;
+    }
+    if (glob) {
+        // A few shots of several width classes run as one launch at the widest one's width when the
+        // device holds them all at once: class after class would take a whole shot's time for each.
+        // (Columns past s add exactly 0, so a shot's results do not depend on the width.)
+        int lo = -1, hi = -1, total = 0;
+        for (int c = 0; c < p.gc.n; ++c) {
+            if (gcnt[c] == 0) continue;
+            if (p.gc.smax[c] > (pio == 0 ? 512 : 1024)) break;  // the general kernel's class stays apart
+            if (lo < 0) lo = c;
+            hi = c;
+            total += gcnt[c];
+        }
+        if (hi > lo) {
+            const int cl = stream_cluster_for(pio, p.gsmax[hi], o->stream_cluster, total, p.full[hi]);
+            const int at_once = cl > 1 ? stream_cluster_capacity_of(pio, p.gsmax[hi] / 32, cl) : p.full[hi];
+            if (total <= at_once && 2 * total < p.full[hi]) {
+                for (int c = lo; c < hi; ++c) gcnt[c] = 0;
+                gcnt[hi] = total;
+                gfirst[hi] = gfirst[lo];
+            }
+        }
+    }
+    CK(cudaMemcpyAsync(dp + L.ctr, hp + L.ctr, L.sdef - L.ctr, cudaMemcpyHostToDevice, st));
+    DecodeArgs a = decode_args(g, ty, reinterpret_cast<const uint32_t*>(dp + L.synd), shots, T, o, dp, dp + L.flags,
+                               reinterpret_cast<int16_t*>(dp + L.iters), reinterpret_cast<unsigned long long*>(dp + L.ctr));
+    const int32_t* const ditems = reinterpret_cast<const int32_t*>(dp + L.items);
+    int32_t* const dcnt = reinterpret_cast<int32_t*>(dp + L.cnt);
+    for (int c = 0; c < kGlobalList; ++c) {
+        if (cnt[c] <= 0) continue;
+        a.list = ditems + first[c];
+        a.list_dir = 1;
+        a.count = dcnt + c;
+        a.next = dcnt + kLists + c;
+        a.tier = list_tier(c);
+        a.max_items = cnt[c];
+        ProfScope ps(g, a.tier, st);
+        CK(launch_decode_list(pio, c, a, g->num_sms, st));
+        ps.end();
+    }
+    if (glob) {
+        a.tier = kGlobalTier;
+        a.gscratch = w.gscratch;
+        a.gscratch_bytes = (int64_t)w.gscratch_bytes;
+        // (a single class has the whole scratch and no neighbour: it runs on `st`)
+        if (p.gc.n == 1) p.need = 0;
+        const int32_t* lists[kMaxGlobalClasses];
+        for (int c = 0; c < kMaxGlobalClasses; ++c) lists[c] = ditems + gfirst[c];
+        int32_t* const dg = dcnt + 2 * kLists;
+        ProfScope ps(g, PROF_GLOBAL, st);
+        const int rc = launch_global_counted(w, a, p, pio, o, gcnt, lists, dg, dg + kMaxGlobalClasses, st);
+        if (rc) return rc;
+        ps.end();
+    }
+    CK(cudaMemcpyAsync(hp, dp, L.cnt, cudaMemcpyDeviceToHost, st));
+    CK(cudaStreamSynchronize(st));
+    const unsigned long long* const ctr = reinterpret_cast<const unsigned long long*>(hp + L.ctr);
+    if (ctr[C_ERRORS]) return fail(BP4M_ECUDA, "decoder kernels rejected shots (internal size check)");
+    const int16_t* const it = reinterpret_cast<const int16_t*>(hp + L.iters);
+    for (int64_t k = 0; k < shots; ++k) {
+        const bool empty = sdef[k] == 0;  // no unsatisfied detector: nothing to decode
+        if (obs_pred) obs_pred[k] = empty ? 0 : hp[k];
+        if (converged) converged[k] = empty || (hp[L.flags + k] & F_CONVERGED) ? 1 : 0;
+        if (iters_used) iters_used[k] = empty ? 0 : it[k];
+    }
+    prof_add_counters(g, ctr);
     return BP4M_OK;
 }
 
@@ -1810,6 +2023,9 @@ static int decode_common(bp4m_graph* g, const uint32_t* syndromes, int64_t shots
             return fail(BP4M_EINVAL, "trace buffers must be device memory");
         if (shots > kBatch) return fail(BP4M_EINVAL, "traced decodes take at most 2^20 shots");
     }
+    if (!tr && !dev_in && shots <= kHostBatch && !is_device_ptr(obs_pred) && !is_device_ptr(converged) &&
+        !is_device_ptr(iters_used))
+        return decode_host(g, g->ws, ty, syndromes, shots, iters, opts, obs_pred, converged, iters_used, st);
     rc = ensure_ws(g, std::max<int64_t>(std::min(kBatch, shots), g->ws.cap));
     if (rc) return rc;
     CK(cudaMemsetAsync(g->ws.ctr, 0, C_NUM * sizeof(unsigned long long), st));
