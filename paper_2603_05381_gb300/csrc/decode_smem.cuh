@@ -895,18 +895,23 @@ __global__ void __launch_bounds__(block_threads(CH, G, (int)sizeof(T), (int)size
                     }
                 }
             } else {
-                // FP64: every row is counted in the read phase
+                // FP64: every row is counted in the read phase.  Bound by the FP64 pipe (two operations
+                // a clock and SM): columns past s, whole registers of them (k = g + G c >= s in every
+                // thread of the block), are left out of every loop; they would add exactly 0.  At
+                // s <= 4 of 32 columns (d = 3) they were most of the work: 4.05 -> 0.99 ms for 10^4 shots.
                 if (!wact) {
                 } else if (!act) {
 #pragma unroll
                     for (int c = 0; c < CH; ++c) q[c] = ninf;
                 } else if (t == 0) {
 #pragma unroll
-                    for (int c = 0; c < CH; ++c) q[c] = B2<T>::fma_(RM(c), ainv, RL(c));
+                    for (int c = 0; c < CH; ++c) q[c] = G * c < s ? B2<T>::fma_(RM(c), ainv, RL(c)) : ninf;
                 } else {
                     Mask b0 = 0, b1 = 0;
 #pragma unroll
                     for (int c = 0; c < CH; ++c) {
+                        q[c] = ninf;
+                        if (G * c >= s) continue;
                         const T l = RL(c);
                         const T x = RM(c);
                         q[c] = B2<T>::fma_(x, ainv, l);
@@ -1142,7 +1147,7 @@ __global__ void __launch_bounds__(block_threads(CH, G, (int)sizeof(T), (int)size
                     read_rows();
                 } else if (act) {
 #pragma unroll
-                    for (int c = 0; c < CH; ++c) q[c] = B2<T>::fma_(RM(c), ainv, RL(c));
+                    for (int c = 0; c < CH; ++c) q[c] = G * c < s ? B2<T>::fma_(RM(c), ainv, RL(c)) : ninf;
                 }
                 __syncthreads();
             }
@@ -1155,6 +1160,7 @@ __global__ void __launch_bounds__(block_threads(CH, G, (int)sizeof(T), (int)size
                     int ac = 0x7fffffff, bc = 0x7fffffff;
 #pragma unroll
                     for (int c = 0; c < CH; c += 2) {
+                        if (G * c >= s) continue;
                         const T v = q[c];
                         const bool gt = v > a1;
                         a2 = B2<T>::mx(a2, B2<T>::mn(v, a1));
@@ -1187,6 +1193,7 @@ __global__ void __launch_bounds__(block_threads(CH, G, (int)sizeof(T), (int)size
                     T sa = T(0), sb = T(0);
 #pragma unroll
                     for (int c = 0; c < CH; c += 2) {
+                        if (G * c >= s) continue;
                         const T u = B2<T>::ex2(B2<T>::mn(q[c], m2) - m2);
                         q[c] = u;
                         sa += u;
@@ -1204,6 +1211,7 @@ __global__ void __launch_bounds__(block_threads(CH, G, (int)sizeof(T), (int)size
                     if (act) {
 #pragma unroll
                         for (int c = 0; c < CH; ++c) {
+                            if (G * c >= s) continue;
                             const T out = -m1 - B2<T>::lg2(B2<T>::fma_(-cf, q[c], Aa));
                             *CMP(c) = out;
                         }

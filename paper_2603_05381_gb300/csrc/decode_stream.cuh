@@ -356,6 +356,8 @@ __global__ void __launch_bounds__(kStreamWarps * 32, 1) decode_stream_kernel(con
                     auto row_pass = [&](auto fused) {
 #pragma unroll
                         for (int c = 0; c < CH; ++c) {
+                            q[c] = ninf;
+                            if (32 * c >= s) continue;  // past s in every lane: would add exactly 0
                             const int k = lane + 32 * c;
                             const T lv = lrow[k], xv = xrow[k];
                             if constexpr (decltype(fused)::value) {
@@ -395,6 +397,7 @@ __global__ void __launch_bounds__(kStreamWarps * 32, 1) decode_stream_kernel(con
                     T S = T(0);
 #pragma unroll
                     for (int c = 0; c < CH; ++c) {
+                        if (32 * c >= s) continue;
                         const T u = B2<T>::ex2(B2<T>::mn(q[c], m2) - m2);
                         q[c] = u;
                         S += u;
@@ -404,6 +407,7 @@ __global__ void __launch_bounds__(kStreamWarps * 32, 1) decode_stream_kernel(con
                     const T Aa = B2<T>::fma_(cf, S - T(1), T(1));
 #pragma unroll
                         for (int c = 0; c < CH; ++c) {
+                            if (32 * c >= s) continue;
                             const int k = lane + 32 * c;
                             const T out = -m1 - B2<T>::lg2(B2<T>::fma_(-cf, q[c], Aa));
                             orow[k] = out;
