@@ -21,8 +21,10 @@ __device__ __forceinline__ uint4 philox4x32_10(uint4 c, uint32_t k0, uint32_t k1
             k0 += 0x9E3779B9u;
             k1 += 0xBB67AE85u;
         }
-        const uint32_t hi0 = __umulhi(0xD2511F53u, c.x), lo0 = 0xD2511F53u * c.x;
-        const uint32_t hi1 = __umulhi(0xCD9E8D57u, c.z), lo1 = 0xCD9E8D57u * c.z;
+        // one wide multiply gives both halves of a product
+        const uint64_t p0 = (uint64_t)0xD2511F53u * c.x, p1 = (uint64_t)0xCD9E8D57u * c.z;
+        const uint32_t hi0 = (uint32_t)(p0 >> 32), lo0 = (uint32_t)p0;
+        const uint32_t hi1 = (uint32_t)(p1 >> 32), lo1 = (uint32_t)p1;
         c = make_uint4(hi1 ^ c.y ^ k0, lo1, hi0 ^ c.w ^ k1, lo0);
     }
     return c;
@@ -35,7 +37,10 @@ __device__ __forceinline__ uint32_t word_of(const uint4& r, int j) {
 constexpr int kSampWarps = 8;
 
 // One warp per shot; lanes take blocks of four units; fired edges XOR into a per-warp
-// shared-memory syndrome.
+// shared-memory syndrome.  Bound by integer issue: ten Philox rounds for four draws.  A block's
+// four thresholds come in one 16-byte load and are compared together; an edge fires in a percent
+// of the draws, so the fired ones of 32 draws are collected and visited in a loop of their own (a
+// branch per draw was taken by some lane of the warp nearly every time).
 __global__ void __launch_bounds__(kSampWarps * 32) sample_circuit_kernel(SampleArgs a) {
     extern __shared__ uint32_t smem_sw[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -50,19 +55,33 @@ __global__ void __launch_bounds__(kSampWarps * 32) sample_circuit_kernel(SampleA
         __syncwarp();
         const uint64_t gs = a.first_shot + (uint64_t)shot;
         uint32_t obs = 0;
-        for (int b = lane; b < n_blocks; b += 32) {
-            const uint4 r = philox4x32_10(make_uint4((uint32_t)gs, (uint32_t)(gs >> 32),
-                                                     (uint32_t)b, a.stream_id), k0, k1);
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const int e = 4 * b + j;
-                if (e < a.n_units && word_of(r, j) < __ldg(a.thr + e)) {
-                    const uint32_t p = __ldg(a.uvo + e);
-                    const int u = (int)(p & 0x7FFFu), v = (int)((p >> 15) & 0x7FFFu);
-                    atomicXor(my + (u >> 5), 1u << (u & 31));
-                    if (v < n_det) atomicXor(my + (v >> 5), 1u << (v & 31));
-                    obs ^= p >> 31;
+        for (int base = 0; base < n_blocks; base += 32 * 8) {
+            // eight blocks a lane: 32 draws, one bit each in `fired`
+            unsigned fired = 0;
+#pragma unroll 4
+            for (int it = 0; it < 8; ++it) {
+                const int b = base + 32 * it + lane;
+                if (b >= n_blocks) break;
+                const uint4 r = philox4x32_10(make_uint4((uint32_t)gs, (uint32_t)(gs >> 32),
+                                                         (uint32_t)b, a.stream_id), k0, k1);
+                uint4 th = make_uint4(0u, 0u, 0u, 0u);  // past the last edge: nothing fires
+                if (4 * b + 3 < a.n_units) {
+                    th = __ldg(reinterpret_cast<const uint4*>(a.thr) + b);
+                } else {
+                    th.x = __ldg(a.thr + 4 * b);
+                    if (4 * b + 1 < a.n_units) th.y = __ldg(a.thr + 4 * b + 1);
+                    if (4 * b + 2 < a.n_units) th.z = __ldg(a.thr + 4 * b + 2);
                 }
+                fired |= ((r.x < th.x ? 1u : 0u) | (r.y < th.y ? 2u : 0u) | (r.z < th.z ? 4u : 0u) | (r.w < th.w ? 8u : 0u)) << (4 * it);
+            }
+            while (fired) {
+                const int bit = __ffs((int)fired) - 1;
+                fired &= fired - 1;
+                const uint32_t p = __ldg(a.uvo + 4 * (base + 32 * (bit >> 2) + lane) + (bit & 3));
+                const int u = (int)(p & 0x7FFFu), v = (int)((p >> 15) & 0x7FFFu);
+                atomicXor(my + (u >> 5), 1u << (u & 31));
+                if (v < n_det) atomicXor(my + (v >> 5), 1u << (v & 31));
+                obs ^= p >> 31;
             }
         }
         __syncwarp();
