@@ -72,6 +72,78 @@ __global__ void finalize_kernel(const uint8_t* flags, int64_t shots, uint8_t* co
 
 }  // namespace
 
+// Streams beside the caller's for the decode lists of one batch, and the events that fork and join
+// them.  Created on first use; one set per workspace.
+constexpr int kLanes = 7;
+struct ListLanes {
+    cudaStream_t st[kLanes] = {};
+    cudaEvent_t fork = nullptr, join[kLanes] = {};
+    void free() {
+        for (int k = 0; k < kLanes; ++k) {
+            if (st[k]) cudaStreamDestroy(st[k]);
+            if (join[k]) cudaEventDestroy(join[k]);
+        }
+        if (fork) cudaEventDestroy(fork);
+        *this = ListLanes();
+    }
+};
+
+// The decode lists of one batch run beside one another.  One after another, each list holds the stream
+// for the slowest of its shots while the other SMs idle: all of a small batch's time, the tails of a
+// large one's.  Measured, one after another -> beside one another (us, T = 50, device batches): 16 / 256 /
+// 4096 / 65536 shots at d = 9 242 / 257 / 582 / 4563 -> 126 / 140 / 404 / 4382; 16 / 1024 at d = 13 616 / 1557
+// -> 238 / 1167; 64 at d = 7 (FP16) 224 -> 134; 16 at d = 5 114 -> 97.  No size measured slower.  Seven lanes
+// and the caller's stream: with three, two calls of 107 and 126 us took 120 and 157.  The lanes are joined on
+// every way out, so that whatever follows on the caller's stream sees the results and may reuse the buffers.
+class ListFan {
+  public:
+    // used(c): list c is launched; `on` = false keeps every launch on `st`
+    template <typename Used>
+    ListFan(ListLanes& lanes, cudaStream_t st, bool on, Used used) : l_(lanes), st_(st) {
+        int lists = 0;
+        for (int c = 0; c < kGlobalList; ++c) lists += used(c) ? 1 : 0;
+        if (!on || lists < 2) return;
+        if (!l_.fork) note(cudaEventCreateWithFlags(&l_.fork, cudaEventDisableTiming));
+        if (err_ == cudaSuccess) note(cudaEventRecord(l_.fork, st));
+        on_ = err_ == cudaSuccess;
+    }
+    ~ListFan() { join(); }
+    ListFan(const ListFan&) = delete;
+    ListFan& operator=(const ListFan&) = delete;
+    // the stream of the next list's launch
+    cudaStream_t next() {
+        const int k = on_ ? launches_++ % (kLanes + 1) - 1 : -1;
+        if (k < 0) return st_;
+        if (k >= forked_) {
+            if (!l_.st[k]) note(cudaStreamCreateWithFlags(&l_.st[k], cudaStreamNonBlocking));
+            if (err_ == cudaSuccess && !l_.join[k]) note(cudaEventCreateWithFlags(&l_.join[k], cudaEventDisableTiming));
+            if (err_ == cudaSuccess) note(cudaStreamWaitEvent(l_.st[k], l_.fork, 0));
+            if (err_ != cudaSuccess) return st_;
+            forked_ = k + 1;
+        }
+        return l_.st[k];
+    }
+    cudaError_t join() {
+        for (int k = 0; k < forked_; ++k) {
+            note(cudaEventRecord(l_.join[k], l_.st[k]));
+            note(cudaStreamWaitEvent(st_, l_.join[k], 0));
+        }
+        forked_ = 0;
+        on_ = false;
+        return err_;
+    }
+
+  private:
+    void note(cudaError_t e) {
+        if (err_ == cudaSuccess) err_ = e;
+    }
+    ListLanes& l_;
+    cudaStream_t st_;
+    bool on_ = false;
+    int forked_ = 0, launches_ = 0;
+    cudaError_t err_ = cudaSuccess;
+};
+
 struct Workspace {
     int64_t cap = 0;
     int n_types = 1;
@@ -94,6 +166,7 @@ struct Workspace {
     int32_t* host_sub = nullptr;  // pinned mirror of the class counts
     cudaStream_t aux = nullptr;   // second stream: classes of few shots run beside the others
     cudaEvent_t ev_sub = nullptr, ev_fork = nullptr, ev_join = nullptr;
+    ListLanes lanes;              // further streams for the decode lists
     cudaEvent_t ev_small = nullptr;
     // staging of small host batches (decode_host): one device block and its pinned mirror
     unsigned char* hb_dev = nullptr;
@@ -347,6 +420,7 @@ void free_ws(Workspace& w) {
     cudaFree(w.subctr);
     cudaFreeHost(w.host_sub);
     if (w.aux) cudaStreamDestroy(w.aux);
+    w.lanes.free();
     if (w.ev_sub) cudaEventDestroy(w.ev_sub);
     if (w.ev_fork) cudaEventDestroy(w.ev_fork);
     if (w.ev_join) cudaEventDestroy(w.ev_join);
@@ -562,6 +636,17 @@ DecodeArgs decode_args(const bp4m_graph* g, int ty, const uint32_t* synd, int64_
     return a;
 }
 
+// A few shots of several width classes run as one launch at the widest one's width when the device
+// holds them all at once: class after class would take a whole shot's time for each.  (Columns past
+// s add exactly 0, so a shot's results do not depend on the width.)  A few shots from
+// device buffers: 14 to 23 at d = 15 0.68-0.72 -> 0.42 ms, 3 to 7 at d = 17 (FP16) 0.8-1.2 -> 0.40 ms.
+bool one_width(const GlobalPlan& p, int pio, const bp4m_opts* o, int widest, int64_t shots) {
+    if (p.gc.smax[widest] > (pio == 0 ? 512 : 1024)) return false;  // the general kernel's class stays apart
+    const int cl = stream_cluster_for(pio, p.gsmax[widest], o->stream_cluster, shots, p.full[widest]);
+    const int at_once = cl > 1 ? stream_cluster_capacity_of(pio, p.gsmax[widest] / 32, cl) : p.full[widest];
+    return shots <= at_once && 2 * shots < p.full[widest];
+}
+
 // Launches the width classes of the global tier whose counts the host knows (class c: host_cnt[c]
 // items at lists[c], device count and work counter at counts[c] and nexts[c]).  A class of fewer
 // shots than half its resident blocks (typically a few shots above the bulk's width) runs on the
@@ -664,12 +749,14 @@ int decode_device(bp4m_graph* g, Workspace& w, int ty, const uint32_t* synd, int
                                                      : "B-BP4MF (FP32) decodes at most 160 unsatisfied checks of a type per shot");
         return BP4M_OK;
     }
-    for (int c = 0; c < kGlobalList; ++c) {
+    // (per-list timing needs the lists one after another)
+    ListFan fan(w.lanes, st, !g->prof_on || tl_no_prof, [&](int c) { return w.host_small[c] > 0; });
+    for (int c = kGlobalList - 1; c >= 0; --c) {  // the slowest shots first
         if (w.host_small[c] <= 0) continue;
         use_list(a, w.lists, shots, w.small, c);
         a.max_items = w.host_small[c];
         ProfScope ps(g, a.tier, st);
-        CK(launch_decode_list(pio, c, a, g->num_sms, st));
+        CK(launch_decode_list(pio, c, a, g->num_sms, fan.next()));
         ps.end();
     }
     const int n_glob = w.host_small[kGlobalList];
@@ -689,11 +776,17 @@ int decode_device(bp4m_graph* g, Workspace& w, int ty, const uint32_t* synd, int
         a.gscratch = w.gscratch;
         a.gscratch_bytes = (int64_t)w.gscratch_bytes;
         ProfScope ps(g, PROF_GLOBAL, st);
-        if (p.gc.n == 1) {
+        const int hi = p.gc.n - 1;  // the widest class: the largest defect count is in it
+        if (hi == 0) {
             a.stream_cl = stream_cluster_for(pio, p.gsmax[0], o->stream_cluster, n_glob, p.full[0]);
             rc = launch_global_classes(a, p, pio, n_glob, w.sub, w.subctr, shots, w.small + kLists + kGlobalList,
                                        g->num_sms, st);
             if (rc) return rc;
+        } else if (one_width(p, pio, o, hi, n_glob)) {
+            a.stream_cl = stream_cluster_for(pio, p.gsmax[hi], o->stream_cluster, n_glob, p.full[hi]);
+            a.gslot_elems = (int64_t)(p.slot_bytes[hi] / (prec == 0 ? sizeof(double) : sizeof(float)) / 3);
+            a.gsmax = p.gsmax[hi];
+            CK(launch_decode_global(pio, a, n_glob, st));
         } else {
             // partition, then read the class counts
             CK(cudaMemsetAsync(w.subctr, 0, 2 * kMaxGlobalClasses * sizeof(int32_t), st));
@@ -708,6 +801,7 @@ int decode_device(bp4m_graph* g, Workspace& w, int ty, const uint32_t* synd, int
         }
         ps.end();
     }
+    CK(fan.join());
     return BP4M_OK;
 }
 
@@ -717,7 +811,7 @@ int decode_device(bp4m_graph* g, Workspace& w, int ty, const uint32_t* synd, int
 // that one copy brings syndromes, lists and zeroed counters, only the lists in use are launched,
 // and one copy takes all results back.  Larger batches are counted on the device: the count of
 // kHostBatch shots costs the host tens of microseconds.  Measured: one d = 5 shot 93 -> 45 us, seven
-// d = 19 shots (one launch for their width classes, below) 875 -> 408 us.
+// d = 19 shots (one launch for their width classes, one_width) 875 -> 408 us.
 constexpr int64_t kHostBatch = 2048;
 
 // One block on both sides: obs, flags, iters and the counters come back; the counters, the lists'
@@ -824,9 +918,6 @@ int decode_host(bp4m_graph* g, Workspace& w, int ty, const uint32_t* synd, int64
         if (rc) return rc;
     }
     if (glob) {
-        // A few shots of several width classes run as one launch at the widest one's width when the
-        // device holds them all at once: class after class would take a whole shot's time for each.
-        // (Columns past s add exactly 0, so a shot's results do not depend on the width.)
         int lo = -1, hi = -1, total = 0;
         for (int c = 0; c < p.gc.n; ++c) {
             if (gcnt[c] == 0) continue;
@@ -835,14 +926,10 @@ int decode_host(bp4m_graph* g, Workspace& w, int ty, const uint32_t* synd, int64
             hi = c;
             total += gcnt[c];
         }
-        if (hi > lo) {
-            const int cl = stream_cluster_for(pio, p.gsmax[hi], o->stream_cluster, total, p.full[hi]);
-            const int at_once = cl > 1 ? stream_cluster_capacity_of(pio, p.gsmax[hi] / 32, cl) : p.full[hi];
-            if (total <= at_once && 2 * total < p.full[hi]) {
-                for (int c = lo; c < hi; ++c) gcnt[c] = 0;
-                gcnt[hi] = total;
-                gfirst[hi] = gfirst[lo];
-            }
+        if (hi > lo && one_width(p, pio, o, hi, total)) {
+            for (int c = lo; c < hi; ++c) gcnt[c] = 0;
+            gcnt[hi] = total;
+            gfirst[hi] = gfirst[lo];
         }
     }
     CK(cudaMemcpyAsync(dp + L.ctr, hp + L.ctr, L.sdef - L.ctr, cudaMemcpyHostToDevice, st));
@@ -850,7 +937,8 @@ int decode_host(bp4m_graph* g, Workspace& w, int ty, const uint32_t* synd, int64
                                reinterpret_cast<int16_t*>(dp + L.iters), reinterpret_cast<unsigned long long*>(dp + L.ctr));
     const int32_t* const ditems = reinterpret_cast<const int32_t*>(dp + L.items);
     int32_t* const dcnt = reinterpret_cast<int32_t*>(dp + L.cnt);
-    for (int c = 0; c < kGlobalList; ++c) {
+    ListFan fan(w.lanes, st, !g->prof_on || tl_no_prof, [&](int c) { return cnt[c] > 0; });
+    for (int c = kGlobalList - 1; c >= 0; --c) {  // the slowest shots first
         if (cnt[c] <= 0) continue;
         a.list = ditems + first[c];
         a.list_dir = 1;
@@ -859,7 +947,7 @@ int decode_host(bp4m_graph* g, Workspace& w, int ty, const uint32_t* synd, int64
         a.tier = list_tier(c);
         a.max_items = cnt[c];
         ProfScope ps(g, a.tier, st);
-        CK(launch_decode_list(pio, c, a, g->num_sms, st));
+        CK(launch_decode_list(pio, c, a, g->num_sms, fan.next()));
         ps.end();
     }
     if (glob) {
@@ -876,6 +964,7 @@ int decode_host(bp4m_graph* g, Workspace& w, int ty, const uint32_t* synd, int64
         if (rc) return rc;
         ps.end();
     }
+    CK(fan.join());
     CK(cudaMemcpyAsync(hp, dp, L.cnt, cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
     const unsigned long long* const ctr = reinterpret_cast<const unsigned long long*>(hp + L.ctr);
@@ -1423,6 +1512,7 @@ struct bp4m_multi {
     bool tuned = false;
     double plan_ms[kPlanCount] = {0, 0, 0};
     int stream_cl = 1;                 // streaming tier's cluster size (autotuner or opts)
+    ListLanes lanes;
     double stream_ms[2] = {0, 0};      // chosen plan with one block per shot / cluster form
     bool use_graph = true;
     cudaGraphExec_t exec = nullptr;
@@ -1450,6 +1540,7 @@ void multi_free(bp4m_multi* m) {
     cudaFree(m->sub);
     cudaFree(m->subctr);
     if (m->exec) cudaGraphExecDestroy(m->exec);
+    m->lanes.free();
     if (m->st) cudaStreamDestroy(m->st);
     delete m;
 }
@@ -1484,10 +1575,11 @@ int multi_enqueue(bp4m_multi* m, const std::vector<int64_t>& shots, int plan, in
     a.stream_cl = stream_cl;
     a.alpha = m->opts.alpha;
     a.ctr = m->ctr;
-    for (int c = 0; c < kGlobalList; ++c) {
+    ListFan fan(m->lanes, st, true, [&](int c) { return tp.used(c); });
+    for (int c = kGlobalList - 1; c >= 0; --c) {  // the slowest shots first
         if (!tp.used(c)) continue;
         use_list(a, m->lists, m->total_cap, m->small, c);
-        CK(launch_decode_list(m->pio, c, a, m->num_sms, st));
+        CK(launch_decode_list(m->pio, c, a, m->num_sms, fan.next()));
     }
     use_list(a, m->lists, m->total_cap, m->small, kGlobalList);
     a.gscratch = m->gscratch;
@@ -1498,6 +1590,7 @@ int multi_enqueue(bp4m_multi* m, const std::vector<int64_t>& shots, int plan, in
                                              m->small + kLists + kGlobalList, m->num_sms, st);
         if (rc) return rc;
     }
+    CK(fan.join());
     for (int k = 0; k < n; ++k) {
         const MultiHostEntry& x = m->e[k];
         if (shots[k] <= 0) continue;

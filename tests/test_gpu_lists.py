@@ -113,3 +113,34 @@ def test_host_requests_match_device_batches(torch, prec, decoder, n):
     only = np.full(n, 77, dtype=np.uint8)
     g.decode_batch(packed, T, opts, None, only, None)
     assert np.array_equal(only, host[1])
+
+
+@pytest.mark.parametrize("prec,decoder,forced", [("fp32", "bp4m", "greedy"), ("fp16", "bp4m", "static"), ("fp32", "bp4mf", "greedy"),
+                                                 ("fp64", "bp4m", "greedy")])
+@pytest.mark.parametrize("sizes", [[1, 9], [7, 15, 23, 31, 47, 63, 79, 95, 111, 127, 143, 159], [30, 161, 200, 257, 330],
+                                   [2, 40, 100, 130, 190, 300, 700]])
+def test_lists_beside_one_another_match_shots_alone(torch, prec, decoder, forced, sizes):
+    # the lists of a batch run on several streams and its few large shots at one width; a shot
+    # alone runs on one stream at its own width.  Two batches follow one another on the caller's
+    # stream, the second over the first's lists, without a wait between them.
+    g, og, _ = _pair(13)
+    T = 6
+    opts = pkg.make_opts(precision=prec, decoder=decoder, forced=forced)
+    n = len(sizes)
+    st = torch.cuda.Stream()
+    runs = []
+    for seed in (35, 36):
+        _, _, synd = _syndromes(torch, og, sizes if seed == 35 else sizes[::-1], seed=seed)
+        runs.append((synd, [torch.full((n,), 77, dtype=t, device="cuda") for t in (torch.uint8, torch.uint8, torch.int16)]))
+    torch.cuda.synchronize()
+    for synd, out in runs:
+        g.decode_batch(synd, T, opts, *out, stream=st.cuda_stream)
+    with torch.cuda.stream(st):
+        got = [[x.clone() for x in out] for _, out in runs]
+    st.synchronize()
+    for (synd, _), out in zip(runs, got):
+        for k in range(n):
+            one = [torch.zeros(1, dtype=t, device="cuda") for t in (torch.uint8, torch.uint8, torch.int16)]
+            g.decode_batch(synd[k:k + 1], T, opts, *one)
+            torch.cuda.synchronize()
+            assert [int(x[k]) for x in out] == [int(x[0]) for x in one], (prec, sizes, k)
