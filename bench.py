@@ -28,14 +28,14 @@ D, P, T = 13, 0.005, 50
 SHOTS = 1_000_000
 SEED = 1
 # FP32 decode kernel of each profile slot (rows per shot, columns per thread CH, threads per row G)
-KERNEL_OF = {"tier1": "decode_smem_kernel<float, CH=32, G=1> (s <= 32)",
-             "tier2": "decode_smem_kernel<float, CH=32, G=2> (s <= 64)",
-             "tier3": "decode_smem_kernel<float, CH=24, G=4> (s <= 96)",
+KERNEL_OF = {"tier1": "decode_small_kernel<float> (s <= 32)",
+             "tier2": "decode_smem_kernel<float, CH=24 and 32, G=2> (s <= 64)",
+             "tier3": "decode_smem_kernel<float, CH=20 and 24, G=4> (s <= 96)",
              "tier4": "decode_smem_kernel<float, CH=28, G=4> (s <= 112)",
              "tier5": "decode_smem_kernel<float, CH=32, G=4> (s <= 128)",
              "tier6": "decode_smem_kernel<float, CH=36, G=4> (s <= 144)",
              "tier7": "decode_smem_kernel<float, CH=40, G=4> (s <= 160)",
-             "global": "decode_stream_kernel<float> (s > 160)"}
+             "global": "decode_wide_kernel<float> (s > 160)"}
 # the 113..144-defect tiers in the register-tile form (--tile-form 2)
 KERNEL_OF_REG = {"tier5": "decode_reg_kernel<NB=32, B=4> (s <= 128)",
                  "tier6": "decode_reg_kernel<NB=24, B=6> (s <= 144)"}
