@@ -16,7 +16,9 @@
  *     cudaPointerGetAttributes.  Host buffers are staged through library-owned device
  *     memory.
  *   - `stream` is a cudaStream_t (NULL = the legacy default stream).  Entry points that
- *     return host-visible results synchronise that stream before returning.
+ *     return host-visible results synchronise that stream before returning.  Work queued in
+ *     it before the call precedes the call's reads and writes of every buffer, host buffers
+ *     included.
  *   - Graphs are owned by the library (bp4m_free_graph releases them).  A graph may be
  *     used by one thread at a time.
  */

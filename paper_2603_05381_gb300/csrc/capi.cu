@@ -172,6 +172,7 @@ struct Workspace {
     unsigned char* hb_dev = nullptr;
     unsigned char* hb_pin = nullptr;
     size_t hb_bytes = 0;
+    cudaEvent_t ev_in = nullptr;  // the work queued before the call (decode_host)
     // B-BP4MF first stage
     int64_t qcap = 0;
     uint8_t* qconv = nullptr;
@@ -427,6 +428,7 @@ void free_ws(Workspace& w) {
     cudaFreeHost(w.host_small);
     cudaFreeHost(w.host_ctr);
     if (w.ev_small) cudaEventDestroy(w.ev_small);
+    if (w.ev_in) cudaEventDestroy(w.ev_in);
     cudaFree(w.hb_dev);
     cudaFreeHost(w.hb_pin);
     cudaFree(w.qconv);
@@ -855,6 +857,13 @@ int decode_host(bp4m_graph* g, Workspace& w, int ty, const uint32_t* synd, int64
     }
     unsigned char* const hp = w.hb_pin;
     unsigned char* const dp = w.hb_dev;
+    // The host reads the rows here, where a copy in the stream would have followed the work queued
+    // before the call (it may still be writing them: pinned rows, or any host memory that the GPU
+    // writes).  An event rather than a wait for the stream: in the legacy stream, or a blocking one,
+    // it also follows the work of the streams that those wait for.  1.2 us where nothing is queued.
+    if (!w.ev_in) CK(cudaEventCreateWithFlags(&w.ev_in, cudaEventDisableTiming));
+    CK(cudaEventRecord(w.ev_in, st));
+    CK(cudaEventSynchronize(w.ev_in));
     std::memset(hp + L.ctr, 0, L.items - L.ctr);
     std::memcpy(hp + L.synd, synd, (size_t)shots * nw * sizeof(uint32_t));
     // defect counts, lists by counting
