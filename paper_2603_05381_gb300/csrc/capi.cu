@@ -39,6 +39,7 @@ int fail(int code, const std::string& msg) {
 
 int cuda_fail(cudaError_t e, const char* where) {
     std::string m = std::string(where) + ": " + cudaGetErrorName(e) + " (" + cudaGetErrorString(e) + ")";
+    (void)cudaGetLastError();  // reported here: the next call's launches ask for the last error
     return fail(e == cudaErrorMemoryAllocation ? BP4M_ENOMEM : BP4M_ECUDA, m);
 }
 

@@ -229,6 +229,7 @@ cudaError_t cudaStreamDestroy(cudaStream_t st) {
     return cudaSuccess;  // (kept allocated: records may name it)
 }
 cudaError_t cudaStreamSynchronize(cudaStream_t s) { LOCK; drain(of(s)); return cudaSuccess; }
+cudaError_t cudaDeviceSynchronize() { LOCK; drain_all(); return cudaSuccess; }
 cudaError_t cudaStreamQuery(cudaStream_t s) { LOCK; return of(s)->q.empty() ? cudaSuccess : cudaErrorNotReady; }
 cudaError_t cudaStreamWaitEvent(cudaStream_t s, cudaEvent_t e, unsigned) {
     LOCK;

@@ -55,3 +55,19 @@ def test_host_rows_are_read_after_the_work_queued_before_the_call(fake, writer, 
     for s in streams.values():
         if s:
             fake.lib.cudaStreamDestroy(s)
+
+
+def test_an_error_of_one_call_does_not_fail_the_next(fake):
+    # the runtime keeps the last error until it is asked for: the next call's launches ask
+    fake.lib.fake_reset()
+    g = fake.graph()
+    rows = fake.syndromes(g, SIZES, seed=4)
+    synd = fake.buffer(rows.size, np.uint32, "device").reshape(rows.shape)
+    synd[:] = rows
+    out = _out(fake, len(SIZES), "device")
+    for k in range(1, 4):
+        fake.lib.fake_fail_launch(k)
+        assert fake.decode(g, synd, out) != 0
+        fake.lib.fake_fail_launch(0)
+        fake.lib.cudaDeviceSynchronize()
+        assert fake.decode(g, synd, out) == 0 and _same(fake, rows, out)
