@@ -60,6 +60,26 @@ bool is_device_ptr(const void* p) {
     return at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged;
 }
 
+// Waits for a call's stream when the call is left with an error: what it has queued may still read
+// the caller's buffers, and the staging and lists that the next call rewrites.
+class WaitOnError {
+  public:
+    explicit WaitOnError(cudaStream_t st) : st_(st) {}
+    ~WaitOnError() {
+        if (!done_) cudaStreamSynchronize(st_);
+    }
+    WaitOnError(const WaitOnError&) = delete;
+    WaitOnError& operator=(const WaitOnError&) = delete;
+    int done() {  // the call ends here, its stream already waited for
+        done_ = true;
+        return BP4M_OK;
+    }
+
+  private:
+    cudaStream_t st_;
+    bool done_ = false;
+};
+
 template <typename T>
 cudaError_t dalloc(T** p, size_t n) {
     return cudaMalloc(reinterpret_cast<void**>(p), std::max<size_t>(n, 1) * sizeof(T));
@@ -661,10 +681,11 @@ int launch_global_counted(Workspace& w, const DecodeArgs& a, const GlobalPlan& p
     const size_t esz = pio == 0 ? sizeof(double) : sizeof(float);
     CK(cudaEventRecord(w.ev_fork, st));
     CK(cudaStreamWaitEvent(w.aux, w.ev_fork, 0));
+    cudaError_t e = cudaSuccess;
     // small classes first, so that their few blocks hold their SMs before the large
     // classes' persistent blocks fill the rest
     for (int pass = 0; pass < 2; ++pass)
-        for (int c = 0; c < p.gc.n; ++c) {
+        for (int c = 0; c < p.gc.n && e == cudaSuccess; ++c) {
             const int cnt = host_cnt[c];
             const bool small = 2 * cnt < p.full[c];
             if (cnt <= 0 || small != (pass == 0)) continue;
@@ -677,10 +698,12 @@ int launch_global_counted(Workspace& w, const DecodeArgs& a, const GlobalPlan& p
             b.gsmax = p.gsmax[c];
             b.stream_cl = stream_cluster_for(pio, b.gsmax, o->stream_cluster, cnt, p.full[c]);
             if (small) b.gscratch = static_cast<unsigned char*>(w.gscratch) + p.need;
-            CK(launch_decode_global(pio, b, small ? cnt : std::min(cnt, p.full[c]), small ? w.aux : st));
+            e = launch_decode_global(pio, b, small ? cnt : std::min(cnt, p.full[c]), small ? w.aux : st);
         }
+    // joined after a failed launch too
     CK(cudaEventRecord(w.ev_join, w.aux));
     CK(cudaStreamWaitEvent(st, w.ev_join, 0));
+    CK(e);
     return BP4M_OK;
 }
 
@@ -856,6 +879,7 @@ int decode_host(bp4m_graph* g, Workspace& w, int ty, const uint32_t* synd, int64
         CK(cudaMallocHost(reinterpret_cast<void**>(&w.hb_pin), b));
         w.hb_bytes = b;
     }
+    WaitOnError wait(st);
     unsigned char* const hp = w.hb_pin;
     unsigned char* const dp = w.hb_dev;
     // The host reads the rows here, where a copy in the stream would have followed the work queued
@@ -987,7 +1011,7 @@ int decode_host(bp4m_graph* g, Workspace& w, int ty, const uint32_t* synd, int64
         if (iters_used) iters_used[k] = empty ? 0 : it[k];
     }
     prof_add_counters(g, ctr);
-    return BP4M_OK;
+    return wait.done();
 }
 
 // B-BP4MF on device-resident syndromes of both types (type 1 = X-checks, type 0 = Z-checks).
@@ -1370,6 +1394,7 @@ int srv_run_batch(bp4m_server* S, SrvSlot& sl, std::vector<SrvPiece>& batch, int
         sl.h_cap = cap;
         sl.h_words = words;
     }
+    WaitOnError wait(st);
     int64_t off = 0;
     for (const SrvPiece& pc : batch) {
         std::memcpy(sl.h_in + (size_t)off * nw, pc.r->synd.data() + (size_t)pc.off * nw, (size_t)pc.cnt * nw * 4);
@@ -1390,7 +1415,7 @@ int srv_run_batch(bp4m_server* S, SrvSlot& sl, std::vector<SrvPiece>& batch, int
                 pc.r->out_conv[pc.off + k] = (uint8_t)(sl.h_out[n + off + k] & F_CONVERGED);
         off += pc.cnt;
     }
-    return BP4M_OK;
+    return wait.done();
 }
 
 void srv_worker(bp4m_server* S, SrvSlot* sl) {
@@ -1877,6 +1902,7 @@ int bp4m_multi_run(bp4m_multi* m, const uint32_t* const* syndromes, const int64_
         if (sh[k] > 0) std::memcpy(m->e[k].h_synd, syndromes[k], (size_t)sh[k] * m->e[k].n_words * 4);
     }
     if (cudaSetDevice(m->device) != cudaSuccess) return fail(BP4M_ECUDA, "cudaSetDevice failed");
+    WaitOnError wait(m->st);
     if (!m->tuned) {
         // autotuner: time every candidate tier plan on this run's shots, keep the fastest
         cudaEvent_t e0, e1;
@@ -1947,7 +1973,7 @@ int bp4m_multi_run(bp4m_multi* m, const uint32_t* const* syndromes, const int64_
     }
     if (m->h_ctr[C_ERRORS])
         return fail(BP4M_EUNSUPPORTED, std::to_string(m->h_ctr[C_ERRORS]) + " shots exceed max_defects unsatisfied detectors");
-    return BP4M_OK;
+    return wait.done();
 }
 
 int bp4m_multi_info(const bp4m_multi* m, bp4m_multi_info_t* out) {
@@ -2131,6 +2157,7 @@ static int decode_common(bp4m_graph* g, const uint32_t* syndromes, int64_t shots
         return decode_host(g, g->ws, ty, syndromes, shots, iters, opts, obs_pred, converged, iters_used, st);
     rc = ensure_ws(g, std::max<int64_t>(std::min(kBatch, shots), g->ws.cap));
     if (rc) return rc;
+    WaitOnError wait(st);
     CK(cudaMemsetAsync(g->ws.ctr, 0, C_NUM * sizeof(unsigned long long), st));
     for (int64_t off = 0; off < shots; off += kBatch) {
         const int64_t nb = std::min(kBatch, shots - off);
@@ -2164,7 +2191,7 @@ static int decode_common(bp4m_graph* g, const uint32_t* syndromes, int64_t shots
     CK(cudaStreamSynchronize(st));
     if (w.host_ctr[C_ERRORS]) return fail(BP4M_ECUDA, "decoder kernels rejected shots (internal size check)");
     prof_add_counters(g, w.host_ctr);
-    return BP4M_OK;
+    return wait.done();
 }
 
 int bp4m_decode_batch(bp4m_graph* g, const uint32_t* syndromes, int64_t shots, int iters,
@@ -2197,6 +2224,7 @@ int bp4m_sample_and_decode_range(bp4m_graph* g, uint64_t first_shot, int64_t sho
     const int64_t cap = std::min(bbp ? kBbpBatch : kBatch, shots);
     rc = ensure_ws(g, std::max<int64_t>(cap, g->ws.cap));
     if (rc) return rc;
+    WaitOnError wait(st);
     Workspace& w = g->ws;
     const int nt = g->host.n_types;
     CK(cudaMemsetAsync(w.ctr, 0, C_NUM * sizeof(unsigned long long), st));
@@ -2231,7 +2259,7 @@ int bp4m_sample_and_decode_range(bp4m_graph* g, uint64_t first_shot, int64_t sho
     if (w.host_ctr[C_ERRORS]) return fail(BP4M_ECUDA, "decoder kernels rejected shots (internal size check)");
     prof_add_counters(g, w.host_ctr);
     fill_counts(w.host_ctr, nt, out);
-    return BP4M_OK;
+    return wait.done();
 }
 
 int bp4m_sample_and_decode(bp4m_graph* g, double p, int64_t shots, uint64_t seed, int iters,
@@ -2282,6 +2310,7 @@ int bp4m_decode_bbp4mf(bp4m_graph* g, const uint32_t* syndromes, int64_t shots, 
     rc = ensure_uploaded(g);
     if (rc) return rc;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
+    WaitOnError wait(st);
     const int nw0 = n_words_of(g, 0), nw1 = n_words_of(g, 1);
     for (int64_t off = 0; off < shots; off += kBbpBatch) {
         const int64_t nb = std::min(kBbpBatch, shots - off);
@@ -2302,7 +2331,7 @@ int bp4m_decode_bbp4mf(bp4m_graph* g, const uint32_t* syndromes, int64_t shots, 
         }
         CK(cudaStreamSynchronize(st));
     }
-    return BP4M_OK;
+    return wait.done();
 }
 
 int bp4m_decode_noalloc(const bp4m_graph* g, const uint32_t* syndromes, int64_t shots, int iters,

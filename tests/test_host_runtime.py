@@ -6,6 +6,7 @@ import numpy as np
 import pytest
 
 from fake_cuda import Fake, build_fake
+from paper_2603_05381_gb300 import _capi
 
 # defect counts: none, every list, and four streaming width classes
 SIZES = [0, 1, 5, 9, 20, 30, 40, 60, 70, 90, 100, 120, 140, 150, 161, 200, 257, 330, 64, 8]
@@ -71,3 +72,60 @@ def test_an_error_of_one_call_does_not_fail_the_next(fake):
         fake.lib.fake_fail_launch(0)
         fake.lib.cudaDeviceSynchronize()
         assert fake.decode(g, synd, out) == 0 and _same(fake, rows, out)
+
+
+@pytest.mark.parametrize("call", ["pageable", "pinned", "device", "sample", "bbp4mf", "fused", "service"])
+def test_a_failed_launch_leaves_no_work_behind(fake, call):
+    # every launch of a call in turn is made to fail: the call returns an error with nothing queued
+    # (its buffers and staging may be used again), and the next call is right
+    lib = fake.lib
+    lib.fake_reset()
+    opts = _capi.Opts(_capi.FP32, 1, 0, 1.0, 0, 0, 0, 0)
+    bbp = call == "bbp4mf"
+    g = fake.graph(5, _capi.CODE_CAPACITY, 0.1) if bbp else fake.graph()
+    n = 60
+    sizes = [k % 9 for k in range(n)] if bbp else [SIZES[(3 * k) % len(SIZES)] for k in range(n)]
+    rows = fake.syndromes(g, sizes, seed=9)
+    where = call if call in ("pageable", "pinned", "device") else "pageable"
+    synd = fake.buffer(rows.size, np.uint32, where).reshape(rows.shape)
+    synd[:] = rows
+    out = _out(fake, n, where)
+    server = multi = None
+    if call == "service":
+        server = lib.bp4m_server_create(1, 64, 0)
+        gid = lib.bp4m_server_add_graph(server, g)
+    if call == "fused":
+        hs, ns = (ctypes.c_void_p * 1)(g.value), (ctypes.c_int64 * 1)(n)
+        multi = lib.bp4m_multi_create(1, hs, None, ns, 5, ctypes.byref(opts), 448, 0)
+        assert multi
+
+    def run():
+        if call == "sample":
+            return lib.bp4m_sample_and_decode_range(g, 0, n, 1, 0, 5, ctypes.byref(opts), ctypes.byref(_capi.Counts()), None)
+        if bbp:
+            two = np.concatenate([rows.ravel(), rows.ravel()])
+            return lib.bp4m_decode_bbp4mf(g, two.ctypes.data, n, 5, ctypes.byref(opts), np.zeros(2 * n, np.uint8).ctypes.data, None, None)
+        if server:
+            r = lib.bp4m_server_submit(server, gid, rows.ctypes.data, n, 5, ctypes.byref(opts), out[0].ctypes.data, out[1].ctypes.data)
+            return lib.bp4m_server_wait(server, r, -1.0, None)
+        if multi:
+            ptr = [(ctypes.c_void_p * 1)(x.ctypes.data) for x in (synd, out[0], out[1])]
+            return lib.bp4m_multi_run(multi, ptr[0], ns, ptr[1], ptr[2])
+        return fake.decode(g, synd, out)
+
+    for k in range(1, 200):
+        lib.fake_fail_launch(k)
+        rc = run()
+        pending = lib.fake_pending()
+        lib.fake_fail_launch(0)
+        if rc == 0:
+            break
+        assert pending == 0, k
+        assert run() == 0 and lib.fake_pending() == 0
+        if call in ("pageable", "pinned", "device"):
+            assert _same(fake, rows, out)
+    assert rc == 0 and k >= (4 if multi else 5)
+    if server:
+        lib.bp4m_server_destroy(server)
+    if multi:
+        lib.bp4m_multi_destroy(multi)
