@@ -116,6 +116,7 @@ struct ListLanes {
 // -> 238 / 1167; 64 at d = 7 (FP16) 224 -> 134; 16 at d = 5 114 -> 97.  No size measured slower.  Seven lanes
 // and the caller's stream: with three, two calls of 107 and 126 us took 120 and 157.  The lanes are joined on
 // every way out, so that whatever follows on the caller's stream sees the results and may reuse the buffers.
+// Where a stream or event cannot be made the lists share those there are, at the least the caller's.
 class ListFan {
   public:
     // used(c): list c is launched; `on` = false keeps every launch on `st`
@@ -124,21 +125,24 @@ class ListFan {
         int lists = 0;
         for (int c = 0; c < kGlobalList; ++c) lists += used(c) ? 1 : 0;
         if (!on || lists < 2) return;
-        if (!l_.fork) note(cudaEventCreateWithFlags(&l_.fork, cudaEventDisableTiming));
-        if (err_ == cudaSuccess) note(cudaEventRecord(l_.fork, st));
-        on_ = err_ == cudaSuccess;
+        if (!l_.fork && !made(cudaEventCreateWithFlags(&l_.fork, cudaEventDisableTiming))) return;
+        note(cudaEventRecord(l_.fork, st));
+        if (err_ == cudaSuccess) lanes_ = kLanes;
     }
     ~ListFan() { join(); }
     ListFan(const ListFan&) = delete;
     ListFan& operator=(const ListFan&) = delete;
     // the stream of the next list's launch
     cudaStream_t next() {
-        const int k = on_ ? launches_++ % (kLanes + 1) - 1 : -1;
+        const int k = launches_++ % (lanes_ + 1) - 1;
         if (k < 0) return st_;
         if (k >= forked_) {
-            if (!l_.st[k]) note(cudaStreamCreateWithFlags(&l_.st[k], cudaStreamNonBlocking));
-            if (err_ == cudaSuccess && !l_.join[k]) note(cudaEventCreateWithFlags(&l_.join[k], cudaEventDisableTiming));
-            if (err_ == cudaSuccess) note(cudaStreamWaitEvent(l_.st[k], l_.fork, 0));
+            if ((!l_.st[k] && !made(cudaStreamCreateWithFlags(&l_.st[k], cudaStreamNonBlocking))) ||
+                (!l_.join[k] && !made(cudaEventCreateWithFlags(&l_.join[k], cudaEventDisableTiming)))) {
+                lanes_ = k;
+                return st_;
+            }
+            note(cudaStreamWaitEvent(l_.st[k], l_.fork, 0));
             if (err_ != cudaSuccess) return st_;
             forked_ = k + 1;
         }
@@ -149,19 +153,22 @@ class ListFan {
             note(cudaEventRecord(l_.join[k], l_.st[k]));
             note(cudaStreamWaitEvent(st_, l_.join[k], 0));
         }
-        forked_ = 0;
-        on_ = false;
+        forked_ = lanes_ = 0;
         return err_;
     }
 
   private:
+    // whether a stream or event was made; if not, its error is not the call's
+    static bool made(cudaError_t e) {
+        if (e != cudaSuccess) (void)cudaGetLastError();
+        return e == cudaSuccess;
+    }
     void note(cudaError_t e) {
         if (err_ == cudaSuccess) err_ = e;
     }
     ListLanes& l_;
     cudaStream_t st_;
-    bool on_ = false;
-    int forked_ = 0, launches_ = 0;
+    int lanes_ = 0, forked_ = 0, launches_ = 0;
     cudaError_t err_ = cudaSuccess;
 };
 
@@ -500,9 +507,13 @@ int ensure_gscratch(Workspace& w, size_t bytes) {
     return BP4M_OK;
 }
 
-// The second stream of the global tier and the events that fork and join it.
+// The second stream of the global tier (left out where it cannot be made) and the events that fork and
+// join it.
 int ensure_aux(Workspace& w) {
-    if (!w.aux) CK(cudaStreamCreateWithFlags(&w.aux, cudaStreamNonBlocking));
+    if (!w.aux && cudaStreamCreateWithFlags(&w.aux, cudaStreamNonBlocking) != cudaSuccess) {
+        w.aux = nullptr;
+        (void)cudaGetLastError();
+    }
     if (!w.ev_fork) CK(cudaEventCreateWithFlags(&w.ev_fork, cudaEventDisableTiming));
     if (!w.ev_join) CK(cudaEventCreateWithFlags(&w.ev_join, cudaEventDisableTiming));
     return BP4M_OK;
@@ -679,8 +690,11 @@ int launch_global_counted(Workspace& w, const DecodeArgs& a, const GlobalPlan& p
                           const int32_t* host_cnt, const int32_t* const* lists, const int32_t* counts, int32_t* nexts,
                           cudaStream_t st) {
     const size_t esz = pio == 0 ? sizeof(double) : sizeof(float);
-    CK(cudaEventRecord(w.ev_fork, st));
-    CK(cudaStreamWaitEvent(w.aux, w.ev_fork, 0));
+    const cudaStream_t aux = w.aux ? w.aux : st;
+    if (aux != st) {
+        CK(cudaEventRecord(w.ev_fork, st));
+        CK(cudaStreamWaitEvent(aux, w.ev_fork, 0));
+    }
     cudaError_t e = cudaSuccess;
     // small classes first, so that their few blocks hold their SMs before the large
     // classes' persistent blocks fill the rest
@@ -698,11 +712,13 @@ int launch_global_counted(Workspace& w, const DecodeArgs& a, const GlobalPlan& p
             b.gsmax = p.gsmax[c];
             b.stream_cl = stream_cluster_for(pio, b.gsmax, o->stream_cluster, cnt, p.full[c]);
             if (small) b.gscratch = static_cast<unsigned char*>(w.gscratch) + p.need;
-            e = launch_decode_global(pio, b, small ? cnt : std::min(cnt, p.full[c]), small ? w.aux : st);
+            e = launch_decode_global(pio, b, small ? cnt : std::min(cnt, p.full[c]), small ? aux : st);
         }
     // joined after a failed launch too
-    CK(cudaEventRecord(w.ev_join, w.aux));
-    CK(cudaStreamWaitEvent(st, w.ev_join, 0));
+    if (aux != st) {
+        CK(cudaEventRecord(w.ev_join, aux));
+        CK(cudaStreamWaitEvent(st, w.ev_join, 0));
+    }
     CK(e);
     return BP4M_OK;
 }

@@ -129,3 +129,21 @@ def test_a_failed_launch_leaves_no_work_behind(fake, call):
         lib.bp4m_server_destroy(server)
     if multi:
         lib.bp4m_multi_destroy(multi)
+
+
+@pytest.mark.parametrize("left", [0, 1, 4, 7])
+@pytest.mark.parametrize("where", ["pageable", "device"])
+def test_a_batch_is_decoded_on_the_streams_there_are(fake, where, left):
+    # no more than `left` further streams can be made: the lists share them, or run on the caller's
+    lib = fake.lib
+    lib.fake_reset()
+    g = fake.new_graph(13)
+    rows = fake.syndromes(g, SIZES, seed=6)
+    synd = fake.buffer(rows.size, np.uint32, where).reshape(rows.shape)
+    synd[:] = rows
+    out = _out(fake, len(SIZES), where)
+    for k in range(2):
+        lib.fake_fail_stream_create(left if k == 0 else -1)
+        assert fake.decode(g, synd, out) == 0, lib.bp4m_last_error()
+        assert _same(fake, rows, out) and lib.fake_list_errors() == 0
+    lib.bp4m_free_graph(g)
