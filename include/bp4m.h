@@ -18,7 +18,8 @@
  *   - `stream` is a cudaStream_t (NULL = the legacy default stream).  Entry points that
  *     return host-visible results synchronise that stream before returning.  Work queued in
  *     it before the call precedes the call's reads and writes of every buffer, host buffers
- *     included.
+ *     included.  Decoding calls run parts of a batch on streams of the library's own beside
+ *     it, of its priority, and join them to it.
  *   - Graphs are owned by the library (bp4m_free_graph releases them).  A graph may be
  *     used by one thread at a time.
  */

@@ -13,6 +13,7 @@
 #include <thread>
 #include <unordered_map>
 #include <cstdio>
+#include <cstdlib>
 #include <cstring>
 #include <new>
 #include <string>
@@ -93,17 +94,32 @@ __global__ void finalize_kernel(const uint8_t* flags, int64_t shots, uint8_t* co
 
 }  // namespace
 
-// Streams beside the caller's for the decode lists of one batch, and the events that fork and join
-// them.  Created on first use; one set per workspace.
+// Streams beside the caller's: for the decode lists of one batch, and for the global tier's classes of few
+// shots.  They have the caller's priority, so that a call ranks as a whole against other streams' work;
+// a set per priority (0 and five above on this GPU), made on first use.  One ListLanes per workspace.
 constexpr int kLanes = 7;
+constexpr int kAuxLane = kLanes;
+constexpr int kLanePrios = 8;
 struct ListLanes {
-    cudaStream_t st[kLanes] = {};
+    cudaStream_t st[kLanePrios][kLanes + 1] = {};
     cudaEvent_t fork = nullptr, join[kLanes] = {};
-    void free() {
-        for (int k = 0; k < kLanes; ++k) {
-            if (st[k]) cudaStreamDestroy(st[k]);
-            if (join[k]) cudaEventDestroy(join[k]);
+    // lane k for a caller's stream; nullptr where it cannot be made, which is not the call's error
+    cudaStream_t lane(cudaStream_t caller, int k) {
+        int prio = 0;
+        if (cudaStreamGetPriority(caller, &prio) != cudaSuccess) (void)cudaGetLastError();
+        cudaStream_t& s = st[std::min(std::abs(prio), kLanePrios - 1)][k];
+        if (!s && cudaStreamCreateWithPriority(&s, cudaStreamNonBlocking, prio) != cudaSuccess) {
+            s = nullptr;
+            (void)cudaGetLastError();
         }
+        return s;
+    }
+    void free() {
+        for (auto& set : st)
+            for (cudaStream_t s : set)
+                if (s) cudaStreamDestroy(s);
+        for (cudaEvent_t e : join)
+            if (e) cudaEventDestroy(e);
         if (fork) cudaEventDestroy(fork);
         *this = ListLanes();
     }
@@ -137,20 +153,20 @@ class ListFan {
         const int k = launches_++ % (lanes_ + 1) - 1;
         if (k < 0) return st_;
         if (k >= forked_) {
-            if ((!l_.st[k] && !made(cudaStreamCreateWithFlags(&l_.st[k], cudaStreamNonBlocking))) ||
-                (!l_.join[k] && !made(cudaEventCreateWithFlags(&l_.join[k], cudaEventDisableTiming)))) {
+            lane_[k] = l_.lane(st_, k);
+            if (!lane_[k] || (!l_.join[k] && !made(cudaEventCreateWithFlags(&l_.join[k], cudaEventDisableTiming)))) {
                 lanes_ = k;
                 return st_;
             }
-            note(cudaStreamWaitEvent(l_.st[k], l_.fork, 0));
+            note(cudaStreamWaitEvent(lane_[k], l_.fork, 0));
             if (err_ != cudaSuccess) return st_;
             forked_ = k + 1;
         }
-        return l_.st[k];
+        return lane_[k];
     }
     cudaError_t join() {
         for (int k = 0; k < forked_; ++k) {
-            note(cudaEventRecord(l_.join[k], l_.st[k]));
+            note(cudaEventRecord(l_.join[k], lane_[k]));
             note(cudaStreamWaitEvent(st_, l_.join[k], 0));
         }
         forked_ = lanes_ = 0;
@@ -158,7 +174,7 @@ class ListFan {
     }
 
   private:
-    // whether a stream or event was made; if not, its error is not the call's
+    // whether an event was made; if not, its error is not the call's
     static bool made(cudaError_t e) {
         if (e != cudaSuccess) (void)cudaGetLastError();
         return e == cudaSuccess;
@@ -168,6 +184,7 @@ class ListFan {
     }
     ListLanes& l_;
     cudaStream_t st_;
+    cudaStream_t lane_[kLanes] = {};
     int lanes_ = 0, forked_ = 0, launches_ = 0;
     cudaError_t err_ = cudaSuccess;
 };
@@ -192,9 +209,8 @@ struct Workspace {
     int32_t* subctr = nullptr;    // counts[kMaxGlobalClasses], next[kMaxGlobalClasses]
     int64_t sub_cap = 0;
     int32_t* host_sub = nullptr;  // pinned mirror of the class counts
-    cudaStream_t aux = nullptr;   // second stream: classes of few shots run beside the others
     cudaEvent_t ev_sub = nullptr, ev_fork = nullptr, ev_join = nullptr;
-    ListLanes lanes;              // further streams for the decode lists
+    ListLanes lanes;              // further streams for the decode lists and the global tier's small classes
     cudaEvent_t ev_small = nullptr;
     // staging of small host batches (decode_host): one device block and its pinned mirror
     unsigned char* hb_dev = nullptr;
@@ -448,7 +464,6 @@ void free_ws(Workspace& w) {
     cudaFree(w.sub);
     cudaFree(w.subctr);
     cudaFreeHost(w.host_sub);
-    if (w.aux) cudaStreamDestroy(w.aux);
     w.lanes.free();
     if (w.ev_sub) cudaEventDestroy(w.ev_sub);
     if (w.ev_fork) cudaEventDestroy(w.ev_fork);
@@ -507,13 +522,8 @@ int ensure_gscratch(Workspace& w, size_t bytes) {
     return BP4M_OK;
 }
 
-// The second stream of the global tier (left out where it cannot be made) and the events that fork and
-// join it.
+// The events that fork and join the global tier's second stream.
 int ensure_aux(Workspace& w) {
-    if (!w.aux && cudaStreamCreateWithFlags(&w.aux, cudaStreamNonBlocking) != cudaSuccess) {
-        w.aux = nullptr;
-        (void)cudaGetLastError();
-    }
     if (!w.ev_fork) CK(cudaEventCreateWithFlags(&w.ev_fork, cudaEventDisableTiming));
     if (!w.ev_join) CK(cudaEventCreateWithFlags(&w.ev_join, cudaEventDisableTiming));
     return BP4M_OK;
@@ -690,7 +700,8 @@ int launch_global_counted(Workspace& w, const DecodeArgs& a, const GlobalPlan& p
                           const int32_t* host_cnt, const int32_t* const* lists, const int32_t* counts, int32_t* nexts,
                           cudaStream_t st) {
     const size_t esz = pio == 0 ? sizeof(double) : sizeof(float);
-    const cudaStream_t aux = w.aux ? w.aux : st;
+    cudaStream_t aux = w.lanes.lane(st, kAuxLane);
+    if (!aux) aux = st;
     if (aux != st) {
         CK(cudaEventRecord(w.ev_fork, st));
         CK(cudaStreamWaitEvent(aux, w.ev_fork, 0));

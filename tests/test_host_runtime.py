@@ -147,3 +147,25 @@ def test_a_batch_is_decoded_on_the_streams_there_are(fake, where, left):
         assert fake.decode(g, synd, out) == 0, lib.bp4m_last_error()
         assert _same(fake, rows, out) and lib.fake_list_errors() == 0
     lib.bp4m_free_graph(g)
+
+
+@pytest.mark.parametrize("where", ["pageable", "device"])
+def test_every_list_has_the_callers_priority(fake, where):
+    lib = fake.lib
+    lib.fake_reset()
+    g = fake.graph()
+    rows = fake.syndromes(g, SIZES, seed=7)
+    synd = fake.buffer(rows.size, np.uint32, where).reshape(rows.shape)
+    synd[:] = rows
+    out = _out(fake, len(SIZES), where)
+    used = set()
+    for prio in (0, -2, -5, 0):
+        st = fake.stream(prio=prio)
+        lib.fake_reset()
+        assert fake.decode(g, synd, out, stream=st) == 0 and _same(fake, rows, out)
+        got = fake.launches()
+        assert np.all(got[:, 3] == prio) and len(set(got[:, 2])) > 5
+        # a priority's streams are made once
+        used |= {(p, s) for p, s in got[:, [3, 2]].tolist() if s != got[0, 2]}
+        lib.cudaStreamDestroy(st)
+    assert len(used) == 3 * 8
