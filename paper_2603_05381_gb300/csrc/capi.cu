@@ -96,7 +96,9 @@ __global__ void finalize_kernel(const uint8_t* flags, int64_t shots, uint8_t* co
 
 // Streams beside the caller's: for the decode lists of one batch, and for the global tier's classes of few
 // shots.  They have the caller's priority, so that a call ranks as a whole against other streams' work;
-// a set per priority (0 and five above on this GPU), made on first use.  One ListLanes per workspace.
+// a set per priority (0 and five above on this GPU), made on first use.  One ListLanes per graph, whose calls
+// follow one another, and per slot of the service, which runs one batch at a time whatever its graph: one
+// per workspace would be eight streams for each slot and graph, of which a slot uses one graph's at a time.
 constexpr int kLanes = 7;
 constexpr int kAuxLane = kLanes;
 constexpr int kLanePrios = 8;
@@ -210,7 +212,7 @@ struct Workspace {
     int64_t sub_cap = 0;
     int32_t* host_sub = nullptr;  // pinned mirror of the class counts
     cudaEvent_t ev_sub = nullptr, ev_fork = nullptr, ev_join = nullptr;
-    ListLanes lanes;              // further streams for the decode lists and the global tier's small classes
+    ListLanes* lanes = nullptr;   // further streams for the decode lists and the global tier's small classes
     cudaEvent_t ev_small = nullptr;
     // staging of small host batches (decode_host): one device block and its pinned mirror
     unsigned char* hb_dev = nullptr;
@@ -249,6 +251,8 @@ struct bp4m_graph {
     int64_t table_bytes = 0;
     bool prepared[4] = {false, false, false, false};
     Workspace ws;
+    ListLanes lanes;  // of this graph's calls and its derived graphs'
+    bp4m_graph() { ws.lanes = &lanes; }
     // measurement: event pairs around every launch while profiling is on
     struct ProfEvent {
         int slot;
@@ -464,7 +468,6 @@ void free_ws(Workspace& w) {
     cudaFree(w.sub);
     cudaFree(w.subctr);
     cudaFreeHost(w.host_sub);
-    w.lanes.free();
     if (w.ev_sub) cudaEventDestroy(w.ev_sub);
     if (w.ev_fork) cudaEventDestroy(w.ev_fork);
     if (w.ev_join) cudaEventDestroy(w.ev_join);
@@ -480,7 +483,9 @@ void free_ws(Workspace& w) {
     cudaFree(w.post);
     cudaFree(w.fsynd);
     cudaFree(w.fbase);
+    ListLanes* const lanes = w.lanes;  // its owner's
     w = Workspace();
+    w.lanes = lanes;
 }
 
 int ensure_ws(bp4m_graph* g, Workspace& w, int64_t cap) {
@@ -700,7 +705,7 @@ int launch_global_counted(Workspace& w, const DecodeArgs& a, const GlobalPlan& p
                           const int32_t* host_cnt, const int32_t* const* lists, const int32_t* counts, int32_t* nexts,
                           cudaStream_t st) {
     const size_t esz = pio == 0 ? sizeof(double) : sizeof(float);
-    cudaStream_t aux = w.lanes.lane(st, kAuxLane);
+    cudaStream_t aux = w.lanes->lane(st, kAuxLane);
     if (!aux) aux = st;
     if (aux != st) {
         CK(cudaEventRecord(w.ev_fork, st));
@@ -803,7 +808,7 @@ int decode_device(bp4m_graph* g, Workspace& w, int ty, const uint32_t* synd, int
         return BP4M_OK;
     }
     // (per-list timing needs the lists one after another)
-    ListFan fan(w.lanes, st, !g->prof_on || tl_no_prof, [&](int c) { return w.host_small[c] > 0; });
+    ListFan fan(*w.lanes, st, !g->prof_on || tl_no_prof, [&](int c) { return w.host_small[c] > 0; });
     for (int c = kGlobalList - 1; c >= 0; --c) {  // the slowest shots first
         if (w.host_small[c] <= 0) continue;
         use_list(a, w.lists, shots, w.small, c);
@@ -998,7 +1003,7 @@ int decode_host(bp4m_graph* g, Workspace& w, int ty, const uint32_t* synd, int64
                                reinterpret_cast<int16_t*>(dp + L.iters), reinterpret_cast<unsigned long long*>(dp + L.ctr));
     const int32_t* const ditems = reinterpret_cast<const int32_t*>(dp + L.items);
     int32_t* const dcnt = reinterpret_cast<int32_t*>(dp + L.cnt);
-    ListFan fan(w.lanes, st, !g->prof_on || tl_no_prof, [&](int c) { return cnt[c] > 0; });
+    ListFan fan(*w.lanes, st, !g->prof_on || tl_no_prof, [&](int c) { return cnt[c] > 0; });
     for (int c = kGlobalList - 1; c >= 0; --c) {  // the slowest shots first
         if (cnt[c] <= 0) continue;
         a.list = ditems + first[c];
@@ -1222,6 +1227,7 @@ struct SrvSlot {
     cudaStream_t st = nullptr;
     std::map<int, Workspace> ws;          // graph id -> workspace
     std::map<int, int64_t> last_use;      // graph id -> batch counter
+    ListLanes lanes;
     uint32_t* h_in = nullptr;             // pinned staging
     uint8_t* h_out = nullptr;             // [2][cap] obs, flags
     int64_t h_cap = 0, h_words = 0;
@@ -1363,6 +1369,7 @@ int srv_run_batch(bp4m_server* S, SrvSlot& sl, std::vector<SrvPiece>& batch, int
     auto it = sl.ws.find(h.graph);
     const size_t before = it == sl.ws.end() ? 0 : ws_bytes(it->second);
     Workspace& w = sl.ws[h.graph];
+    w.lanes = &sl.lanes;
     sl.last_use[h.graph] = stamp;
     // per-shot buffers are sized for a full batch at once: a workspace that grew request by
     // request would free and reallocate device memory (a device-wide synchronisation that
@@ -1816,6 +1823,7 @@ int bp4m_server_destroy(bp4m_server* S) {
         if (sl->th.joinable()) sl->th.join();
     for (SrvSlot* sl : S->slots) {
         for (auto& kv : sl->ws) free_ws(kv.second);
+        sl->lanes.free();
         cudaFreeHost(sl->h_in);
         cudaFreeHost(sl->h_out);
         if (sl->st) cudaStreamDestroy(sl->st);
@@ -2316,6 +2324,7 @@ int bp4m_sample_and_decode(bp4m_graph* g, double p, int64_t shots, uint64_t seed
         }
     }
     g->derived.push_back(dg);
+    dg->ws.lanes = g->ws.lanes;  // one call at a time uses either
     if (dg->prof_on != g->prof_on) {
         prof_clear(dg);
         dg->prof_on = g->prof_on;
@@ -2516,6 +2525,7 @@ void bp4m_free_graph(bp4m_graph* g) {
         }
         free_ws(g->ws);
     }
+    g->lanes.free();  // (derived graphs may have used them where this one was not uploaded)
     delete g;
 }
 

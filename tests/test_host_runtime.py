@@ -169,3 +169,54 @@ def test_every_list_has_the_callers_priority(fake, where):
         used |= {(p, s) for p, s in got[:, [3, 2]].tolist() if s != got[0, 2]}
         lib.cudaStreamDestroy(st)
     assert len(used) == 3 * 8
+
+
+def test_streams_of_a_service_belong_to_its_slots(fake):
+    # a slot decodes one batch at a time: its streams serve every graph it meets
+    lib = fake.lib
+    lib.fake_reset()
+    opts = _capi.Opts(_capi.FP32, 1, 0, 1.0, 0, 0, 0, 0)
+    graphs = [fake.graph(13), fake.graph(11), fake.graph(9), fake.graph(7)]
+    sizes = [1, 9, 20, 30, 40, 60, 70, 90]
+    rows = [fake.syndromes(g, sizes, seed=8) for g in graphs]
+    before, slots = lib.fake_streams(), 2
+    server = lib.bp4m_server_create(slots, 64, 0)
+    ids = [lib.bp4m_server_add_graph(server, g) for g in graphs]
+    for _ in range(6):
+        reqs = []
+        for gid, r in zip(ids, rows):
+            out = [np.zeros(len(sizes), np.uint8) for _ in range(2)]
+            reqs.append((lib.bp4m_server_submit(server, gid, r.ctypes.data, len(sizes), 5, ctypes.byref(opts), out[0].ctypes.data,
+                                                out[1].ctypes.data), r, out))
+        for rid, r, out in reqs:
+            assert lib.bp4m_server_wait(server, rid, -1.0, None) == 0
+            assert all(np.array_equal(a, b) for a, b in zip(out, Fake.expected(r)[:2]))
+    assert lib.fake_max_streams() <= before + slots * (1 + 8)
+    lib.bp4m_server_destroy(server)
+    assert lib.fake_streams() == before
+
+
+def test_a_graphs_streams_outlive_its_workspace(fake):
+    # larger batches and other error rates reuse the streams
+    lib = fake.lib
+    lib.fake_reset()
+    g = fake.new_graph(5)
+    before = lib.fake_streams()
+    opts = _capi.Opts(_capi.FP32, 1, 0, 1.0, 0, 0, 0, 0)
+    for n in (30, 300, 3000):
+        rows = fake.syndromes(g, [(5 * k) % 60 for k in range(n)], seed=n)
+        synd = fake.buffer(rows.size, np.uint32, "device").reshape(rows.shape)
+        synd[:] = rows
+        out = _out(fake, n, "device")
+        assert fake.decode(g, synd, out) == 0 and _same(fake, rows, out)
+    for p in (0.004, 0.006):
+        assert lib.bp4m_sample_and_decode(g, p, 300, 1, 5, ctypes.byref(opts), ctypes.byref(_capi.Counts()), None) == 0
+    used = set(fake.launches()[:, 2].tolist())
+    assert lib.fake_streams() - before <= 8 and len(used) <= 9
+    lib.bp4m_free_graph(g)
+    assert lib.fake_streams() == before
+    # a graph of which only another error rate's was used
+    g = fake.new_graph(5)
+    assert lib.bp4m_sample_and_decode(g, 0.004, 300, 1, 5, ctypes.byref(opts), ctypes.byref(_capi.Counts()), None) == 0
+    lib.bp4m_free_graph(g)
+    assert lib.fake_streams() == before
