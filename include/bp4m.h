@@ -243,8 +243,8 @@ int bp4m_sample_and_decode_range(bp4m_graph* g, uint64_t first_shot, int64_t sho
    (negative weight, a case the paper does not treat) is taken as present, as matching
    decoders with negative weights do: its endpoints flip in the shot's syndrome, its
    observable bit is added to the output, and it weighs as its complement.  Every edge then
-   weighs max(|ln((1-P)/P)|, 2^-20), Dijkstra from every unsatisfied check of the flipped
-   syndrome yields the shot's priors, and BP4MF (alpha from opts) runs for `iters`
+   weighs max(|ln((1-P)/P)|, 2^-20), the shortest paths from every unsatisfied check of the flipped
+   syndrome yield the shot's priors, and BP4MF (alpha from opts) runs for `iters`
    iterations.  At most 160 (FP32) or 112 (FP64) unsatisfied checks
    of a type per shot (BP4M_EUNSUPPORTED beyond).  syndromes: uint32 [2][shots][n_words] (type 0 then type 1, the layout of
    bp4m_sample); outputs obs_pred and flags (bit0 converged, bit3 first stage): uint8

@@ -182,7 +182,6 @@ template <typename MS, typename T>
 struct MsgIO {
     static __device__ __forceinline__ T ld(const MS* p) { return *p; }
     static __device__ __forceinline__ void st(MS* p, T v) { *p = v; }
-    static __device__ __forceinline__ T zero_store() { return T(0); }
 };
 
 template <>
@@ -251,14 +250,6 @@ template <typename T, int N>
 struct Regs {
     T v[N];
     __device__ __forceinline__ T& operator[](int c) { return v[c]; }
-    // runtime column index: a select chain, so that the array stays in registers
-    __device__ __forceinline__ T get(int c) const {
-        T r = T(0);
-#pragma unroll
-        for (int k = 0; k < N; ++k)
-            if (k == c) r = v[k];
-        return r;
-    }
 };
 
 template <int N>
@@ -266,13 +257,6 @@ struct Regs<float, N> {
     static_assert(N % 2 == 0, "FP32 rows are cached in column pairs");
     float2 p[N / 2];
     __device__ __forceinline__ float& operator[](int c) { return (c & 1) ? p[c >> 1].y : p[c >> 1].x; }
-    __device__ __forceinline__ float get(int c) const {
-        float r = 0.f;
-#pragma unroll
-        for (int k = 0; k < N; ++k)
-            if (k == c) r = (k & 1) ? p[k >> 1].y : p[k >> 1].x;
-        return r;
-    }
 };
 
 // min(u, 1) for u >= 0 (saturate), on the FMA pipe: the leave-one-out sum takes the row's
@@ -341,8 +325,8 @@ __host__ __device__ constexpr int block_threads(int ch, int g, int elem_bytes, i
 }
 
 // RW = true: the B-BP4MF second stage.  The shot's priors, pair weights and parities are
-// computed in the block by Dijkstra from every defect over per-qubit weights derived from
-// the first stage's posteriors (instead of being gathered from the static tables).
+// computed in the block from the shortest paths of every defect over per-qubit weights derived
+// from the first stage's posteriors (instead of being gathered from the static tables).
 template <typename T, int CH, int G, bool TRACE, bool RW = false, typename MS = T>
 __global__ void __launch_bounds__(block_threads(CH, G, (int)sizeof(T), (int)sizeof(MS), RW), blocks_for(CH * G * G, (int)sizeof(T), (int)sizeof(MS))) decode_smem_kernel(const DecodeArgs a) {
     constexpr int SMAX = CH * G;
@@ -370,8 +354,8 @@ __global__ void __launch_bounds__(block_threads(CH, G, (int)sizeof(T), (int)size
     float* const nrefv = reinterpret_cast<float*>(smem + nref_offset<T, MS>(SMAX, G, HELP));
     // static-partition forced convergence: factors in processing order
     short* order = reinterpret_cast<short*>(smem + nref_offset<T, MS>(SMAX, G, HELP) + (HALF ? (size_t)SMAX * 4 : 0));
-    // RW only: per-shot W (FP64) and parity over local ranks, Dijkstra state per warp, in
-    // this block's global scratch slot (layout of rw_slot_layout)
+    // RW only: per-shot W (FP64) and parity over local ranks, distances and predecessors per warp
+    // and the weight of each qubit, in this block's global scratch slot (layout of rw_slot_layout)
     const int rw_nodes = a.tb.n_det + 1;
     unsigned char* rw_slot = RW ? reinterpret_cast<unsigned char*>(a.gscratch) + (size_t)blockIdx.x * a.rw_slot_bytes
                                 : nullptr;

@@ -94,7 +94,6 @@ struct DecodeArgs {
     int decoder = 0;                 // 0 = BP4M, 1 = BP4MF
     int forced_static = 0;           // forced convergence: 0 = global greedy, 1 = static partition
     double alpha = 1.0;
-    int pitch = 0;                   // shared-memory row pitch in elements
     int tier = 0;                    // decode tier (per-tier counters)
     // outputs (any may be null)
     uint8_t* obs_pred = nullptr;
@@ -110,12 +109,12 @@ struct DecodeArgs {
     int64_t count_val = 0;
     int* err_flag = nullptr;         // set to 1 by a block that meets a shot it cannot hold
     int flags_mode = 0;              // 0: `flags` gets F_* bits; 1: `flags` gets converged 0/1
-    // B-BP4MF second stage: the shot's priors come from Dijkstra over per-qubit weights
+    // B-BP4MF second stage: the shot's priors come from shortest paths over per-qubit weights
     // max(ln((1-P)/P), kRwMinWeight), P = the first stage's posterior (rw_post
     // [shots][n_units]); adjacency in CSR over n_det + 1 nodes, entries packed
     // neighbour | unit << 15 | obs << 31, each node's entries sorted by (neighbour, obs).
-    // Per-shot W, parity and Dijkstra state live in a per-block slot of gscratch of
-    // rw_slot_bytes bytes (rw_scratch_bytes()).
+    // Per-shot W, parity, distances, predecessors and the qubits' weights live in a per-block
+    // slot of gscratch of rw_slot_bytes bytes (rw_scratch_bytes()).
     const double* rw_post = nullptr;
     const int* rw_off = nullptr;
     const uint32_t* rw_adj = nullptr;

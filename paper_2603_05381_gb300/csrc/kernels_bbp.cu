@@ -170,7 +170,7 @@ __global__ void __launch_bounds__(kQbpThreads) qbp_kernel(QbpArgs a) {
 }
 
 // Second-stage preparation.  The paper does not say how an edge whose posterior P exceeds
-// 1/2 (weight ln((1-P)/P) < 0, no shortest paths) enters Dijkstra's algorithm; as matching
+// 1/2 (weight ln((1-P)/P) < 0, no shortest paths) enters the shortest-path search; as matching
 // decoders with negative weights do, such an edge is taken as present: its endpoints flip in
 // a copy of the syndrome, its observable bit goes into a base parity added to the decoded
 // one, and it enters the graph with probability 1 - P.  One warp per (type, shot).
