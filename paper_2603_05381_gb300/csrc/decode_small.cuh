@@ -526,15 +526,20 @@ __global__ void __launch_bounds__(kSmallWarps * 32, small_blocks(LG)) decode_sma
         if (live) ++t;
         __syncwarp();
     }
-    __syncwarp();
-    if (i == 0 && a.ctr) {
-        atomicAdd(a.ctr + C_ITERS, acc[0]);
-        atomicAdd(a.ctr + C_MSGS, acc[1]);
-        atomicAdd(a.ctr + C_DEFECTS, acc[2]);
-        atomicAdd(a.ctr + C_TIER_MSGS + a.tier, acc[1]);
-        atomicAdd(a.ctr + C_TIER_SHOTS + a.tier, acc[3]);
-        atomicAdd(a.ctr + C_FC_RUNS, acc[4]);
-        atomicAdd(a.ctr + C_FC_ROUNDS, acc[5]);
+    // The block's sums: one addition a counter, none where nothing was decoded.  (One a counter and group was
+    // 136,000 additions to seven addresses in an 8-row launch, 70 us whatever its shots: a fused run of one
+    // d = 5 code-capacity shot took 161 us, 72 now.)
+    __syncthreads();
+    if (threadIdx.x < 6 && a.ctr) {
+        const int k = threadIdx.x;
+        unsigned long long v = 0;
+        for (int w = 0; w < kSmallWarps; ++w)
+            for (int q = 0; q < NG; ++q) v += sh_acc[w][q][k];
+        if (v) {
+            const int slot = k == 0 ? C_ITERS : k == 1 ? C_MSGS : k == 2 ? C_DEFECTS : k == 3 ? C_TIER_SHOTS + a.tier : k == 4 ? C_FC_RUNS : C_FC_ROUNDS;
+            atomicAdd(a.ctr + slot, v);
+            if (k == 1) atomicAdd(a.ctr + C_TIER_MSGS + a.tier, v);
+        }
     }
 }
 

@@ -1234,7 +1234,7 @@ __global__ void __launch_bounds__(block_threads(CH, G, (int)sizeof(T), (int)size
         if constexpr (HELP) pb ^= 1;
         __syncthreads();
     }
-    if (tid == 0 && a.ctr) {
+    if (tid == 0 && a.ctr && acc_shots) {
         atomicAdd(a.ctr + C_ITERS, acc_it);
         atomicAdd(a.ctr + C_MSGS, acc_msg);
         atomicAdd(a.ctr + C_DEFECTS, acc_def);

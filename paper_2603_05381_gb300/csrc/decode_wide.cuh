@@ -789,7 +789,7 @@ __global__ void __launch_bounds__(WideShape<CH, MS, CL>::W * 32, WideShape<CH, M
         }
         __syncthreads();
     }
-    if (tid == 0 && crank == 0 && a.ctr) {
+    if (tid == 0 && crank == 0 && a.ctr && acc_shots) {
         atomicAdd(a.ctr + C_ITERS, acc_it);
         atomicAdd(a.ctr + C_MSGS, acc_msg);
         atomicAdd(a.ctr + C_DEFECTS, acc_def);
