@@ -867,10 +867,13 @@ int decode_device(bp4m_graph* g, Workspace& w, int ty, const uint32_t* synd, int
 // about 10; the rest went into launches for empty lists, a wait for the counts, and a pageable
 // copy per buffer.  The host counts the defects while it stages the syndromes in pinned memory, so
 // that one copy brings syndromes, lists and zeroed counters, only the lists in use are launched,
-// and one copy takes all results back.  Larger batches are counted on the device: the count of
-// kHostBatch shots costs the host tens of microseconds.  Measured: one d = 5 shot 93 -> 45 us, seven
-// d = 19 shots (one launch for their width classes, one_width) 875 -> 408 us.
-constexpr int64_t kHostBatch = 2048;
+// and one copy takes all results back.  Larger batches are counted on the device: by then the host's
+// count of the rows takes longer than the launches and waits that it saves.  Measured, device against
+// host (us): one d = 5 shot 95 / 42; 37 words a row (d = 13) 200, 1000 and 2048 shots 111 / 63, 125 / 94 and 133 / 129;
+// 81 words (d = 17) 700, 1000 and 1400 shots 133 / 106, 138 / 129 and 136 / 156; 152 words (d = 21) 400, 700 and 2048 shots
+// 141 / 115, 139 / 151 and 149 / 303.  Seven d = 19 shots (one launch for their width classes, one_width) 875 -> 408.
+constexpr int64_t kHostBatch = 2048;    // shots
+constexpr int64_t kHostWords = 65536;  // syndrome words
 
 // One block on both sides: obs, flags, iters and the counters come back; the counters, the lists'
 // counts and work counters, the items and the syndromes go up.
@@ -2187,7 +2190,7 @@ static int decode_common(bp4m_graph* g, const uint32_t* syndromes, int64_t shots
             return fail(BP4M_EINVAL, "trace buffers must be device memory");
         if (shots > kBatch) return fail(BP4M_EINVAL, "traced decodes take at most 2^20 shots");
     }
-    if (!tr && !dev_in && shots <= kHostBatch && !is_device_ptr(obs_pred) && !is_device_ptr(converged) &&
+    if (!tr && !dev_in && shots <= kHostBatch && shots * nw <= kHostWords && !is_device_ptr(obs_pred) && !is_device_ptr(converged) &&
         !is_device_ptr(iters_used))
         return decode_host(g, g->ws, ty, syndromes, shots, iters, opts, obs_pred, converged, iters_used, st);
     rc = ensure_ws(g, std::max<int64_t>(std::min(kBatch, shots), g->ws.cap));

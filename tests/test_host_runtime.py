@@ -5,7 +5,7 @@ import ctypes
 import numpy as np
 import pytest
 
-from fake_cuda import Fake, build_fake
+from fake_cuda import CLASSIFY, Fake, build_fake
 from paper_2603_05381_gb300 import _capi
 
 # defect counts: none, every list, and four streaming width classes
@@ -220,3 +220,16 @@ def test_a_graphs_streams_outlive_its_workspace(fake):
     assert lib.bp4m_sample_and_decode(g, 0.004, 300, 1, 5, ctypes.byref(opts), ctypes.byref(_capi.Counts()), None) == 0
     lib.bp4m_free_graph(g)
     assert lib.fake_streams() == before
+
+
+@pytest.mark.parametrize("d,n,on_host", [(3, 2048, True), (3, 2049, False), (13, 1700, True), (13, 1800, False)])
+def test_host_counts_small_batches_only(fake, d, n, on_host):
+    # at most 2048 shots and 65,536 words of rows (37 a row at d = 13): beyond that the host's count
+    # takes longer than the launches it saves
+    lib = fake.lib
+    lib.fake_reset()
+    g = fake.graph(d)
+    rows = fake.syndromes(g, [k % 9 for k in range(n)], seed=n)
+    out = _out(fake, n, "pageable")
+    assert fake.decode(g, rows, out) == 0 and _same(fake, rows, out)
+    assert (CLASSIFY not in fake.launches()[:, 0]) == on_host
