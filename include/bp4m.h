@@ -285,7 +285,10 @@ int bp4m_decode_noalloc(const bp4m_graph* g, const uint32_t* syndromes, int64_t 
    algorithmic message updates of each decoding tier are counted.  Enabling resets the
    accumulators; reading synchronises the events.  Slots: 0 = defect classification,
    1..7 = shared-memory decode tiers (s <= 32, 64, 96, 112, 128, 144, 160 in FP32; 32, 64,
-   112 in FP64), 8 = global-memory decode tier, 9 = sampler, 10 = failure counting. */
+   112 in FP64), 8 = global-memory decode tier, 9 = sampler, 10 = failure counting.
+   While enabled, the decode lists of a batch run one after another, so that each has a time of
+   its own; otherwise they run beside one another, so the times add up to more than an unprofiled
+   call's.  (Small host batches are counted on the host and have no classification launch.) */
 #define BP4M_PROF_SLOTS 11
 typedef struct {
     int64_t launches[BP4M_PROF_SLOTS];
