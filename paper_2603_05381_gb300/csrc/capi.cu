@@ -588,7 +588,7 @@ int launch_global_classes(DecodeArgs a, const GlobalPlan& p, int prec, int64_t i
         a.next = next_single;
         a.gslot_elems = (int64_t)(p.slot_bytes[0] / esz / 3);
         a.gsmax = p.gsmax[0];
-        CK(launch_decode_global(prec, a, (int)std::min<int64_t>(items, p.full[0]), st));
+        CK(launch_decode_global(prec, a, (int)std::min<int64_t>(items, p.full[0]), num_sms, st));
         return BP4M_OK;
     }
     CK(cudaMemsetAsync(w_subctr, 0, 2 * kMaxGlobalClasses * sizeof(int32_t), st));
@@ -600,7 +600,7 @@ int launch_global_classes(DecodeArgs a, const GlobalPlan& p, int prec, int64_t i
         b.next = w_subctr + kMaxGlobalClasses + c;
         b.gslot_elems = (int64_t)(p.slot_bytes[c] / esz / 3);
         b.gsmax = p.gsmax[c];
-        CK(launch_decode_global(prec, b, (int)std::min<int64_t>(items, p.full[c]), st));
+        CK(launch_decode_global(prec, b, (int)std::min<int64_t>(items, p.full[c]), num_sms, st));
     }
     return BP4M_OK;
 }
@@ -703,7 +703,7 @@ bool one_width(const GlobalPlan& p, int pio, const bp4m_opts* o, int widest, int
 // whole shot's decode on a few SMs; empty classes are skipped.
 int launch_global_counted(Workspace& w, const DecodeArgs& a, const GlobalPlan& p, int pio, const bp4m_opts* o,
                           const int32_t* host_cnt, const int32_t* const* lists, const int32_t* counts, int32_t* nexts,
-                          cudaStream_t st) {
+                          int num_sms, cudaStream_t st) {
     const size_t esz = pio == 0 ? sizeof(double) : sizeof(float);
     cudaStream_t aux = w.lanes->lane(st, kAuxLane);
     if (!aux) aux = st;
@@ -728,7 +728,7 @@ int launch_global_counted(Workspace& w, const DecodeArgs& a, const GlobalPlan& p
             b.gsmax = p.gsmax[c];
             b.stream_cl = stream_cluster_for(pio, b.gsmax, o->stream_cluster, cnt, p.full[c]);
             if (small) b.gscratch = static_cast<unsigned char*>(w.gscratch) + p.need;
-            e = launch_decode_global(pio, b, small ? cnt : std::min(cnt, p.full[c]), small ? aux : st);
+            e = launch_decode_global(pio, b, small ? cnt : std::min(cnt, p.full[c]), num_sms, small ? aux : st);
         }
     // joined after a failed launch too
     if (aux != st) {
@@ -844,7 +844,7 @@ int decode_device(bp4m_graph* g, Workspace& w, int ty, const uint32_t* synd, int
             a.stream_cl = stream_cluster_for(pio, p.gsmax[hi], o->stream_cluster, n_glob, p.full[hi]);
             a.gslot_elems = (int64_t)(p.slot_bytes[hi] / (prec == 0 ? sizeof(double) : sizeof(float)) / 3);
             a.gsmax = p.gsmax[hi];
-            CK(launch_decode_global(pio, a, n_glob, st));
+            CK(launch_decode_global(pio, a, n_glob, g->num_sms, st));
         } else {
             // partition, then read the class counts
             CK(cudaMemsetAsync(w.subctr, 0, 2 * kMaxGlobalClasses * sizeof(int32_t), st));
@@ -854,7 +854,7 @@ int decode_device(bp4m_graph* g, Workspace& w, int ty, const uint32_t* synd, int
             CK(cudaEventSynchronize(w.ev_sub));
             const int32_t* lists[kMaxGlobalClasses];
             for (int c = 0; c < p.gc.n; ++c) lists[c] = w.sub + (size_t)c * shots;
-            rc = launch_global_counted(w, a, p, pio, o, w.host_sub, lists, w.subctr, w.subctr + kMaxGlobalClasses, st);
+            rc = launch_global_counted(w, a, p, pio, o, w.host_sub, lists, w.subctr, w.subctr + kMaxGlobalClasses, g->num_sms, st);
             if (rc) return rc;
         }
         ps.end();
@@ -1029,7 +1029,7 @@ int decode_host(bp4m_graph* g, Workspace& w, int ty, const uint32_t* synd, int64
         for (int c = 0; c < kMaxGlobalClasses; ++c) lists[c] = ditems + gfirst[c];
         int32_t* const dg = dcnt + 2 * kLists;
         ProfScope ps(g, PROF_GLOBAL, st);
-        const int rc = launch_global_counted(w, a, p, pio, o, gcnt, lists, dg, dg + kMaxGlobalClasses, st);
+        const int rc = launch_global_counted(w, a, p, pio, o, gcnt, lists, dg, dg + kMaxGlobalClasses, g->num_sms, st);
         if (rc) return rc;
         ps.end();
     }

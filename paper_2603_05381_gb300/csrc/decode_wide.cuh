@@ -67,13 +67,18 @@ constexpr size_t wide_slot_bytes(int ld) {
 // 16-bit messages at 448 and 512 columns: 16.2 -> 17.2 us, so one).
 constexpr int wide_blocks(int ch, int msg_bytes) { return ch <= (msg_bytes == 4 ? 16 : 12) ? 2 : 1; }
 
-template <int CH, typename MS, int CL = 1>
+// ALONE: one block per SM with the warps of two, for launches of no more shots than SMs.  Blocks of half
+// the warps would leave half of an SM idle, or meet two to an SM while other SMs hold the batch's smaller
+// classes.  FP32, halves -> alone (us, BP4M at T = 12 / BP4MF at T = 10): 152 shots of 192 columns
+// 243 / 633 -> 230 / 580, of 320 674 / 1866 -> 584 / 1419, of 448 1320 / 4996 -> 1152 / 3166, of 512 1672 / 6440 ->
+// 1460 / 4598; one shot of 448 columns 848 / 2685 -> 729 / 1976.
+template <int CH, typename MS, int CL = 1, bool ALONE = false>
 struct WideShape {
     static constexpr int LD = 32 * CH;
     static constexpr bool HALF = sizeof(MS) == 2;
     // output stage pitch in elements: row pairs of a column pair in distinct banks
     static constexpr int SP = LD + 2;
-    static constexpr int blocks = CL == 1 ? wide_blocks(CH, (int)sizeof(MS)) : 1;
+    static constexpr int blocks = CL == 1 && !ALONE ? wide_blocks(CH, (int)sizeof(MS)) : 1;
     // prefetched message rows: 16-bit rows apart by half the banks
     static constexpr int PX = HALF ? LD + 32 : LD;
     static constexpr size_t per_warp = 2 * ((size_t)LD * 4 + (size_t)(PX + SP) * sizeof(MS));
@@ -107,9 +112,9 @@ struct WideShape {
     static constexpr size_t slot_bytes = wide_slot_bytes<MS>(LD);
 };
 
-template <int CH, typename MS, int CL>
-__global__ void __launch_bounds__(WideShape<CH, MS, CL>::W * 32, WideShape<CH, MS, CL>::blocks) decode_wide_kernel(const DecodeArgs a) {
-    using SH = WideShape<CH, MS, CL>;
+template <int CH, typename MS, int CL, bool ALONE = false>
+__global__ void __launch_bounds__(WideShape<CH, MS, CL, ALONE>::W * 32, WideShape<CH, MS, CL, ALONE>::blocks) decode_wide_kernel(const DecodeArgs a) {
+    using SH = WideShape<CH, MS, CL, ALONE>;
     using IO = MsgIO<MS, float>;
     constexpr bool HALF = SH::HALF;
     constexpr int LD = SH::LD, SP = SH::SP, PX = SH::PX, W = SH::W, RB = SH::RB, NTH = W * 32;
@@ -812,14 +817,22 @@ __global__ void __launch_bounds__(WideShape<CH, MS, CL>::W * 32, WideShape<CH, M
 }
 
 
-template <int CH, typename MS>
-cudaError_t run_wide(const DecodeArgs& a, int slots, cudaStream_t st) {
-    using SH = WideShape<CH, MS>;
-    auto kern = decode_wide_kernel<CH, MS, 1>;
+template <int CH, typename MS, bool ALONE>
+cudaError_t run_wide1(const DecodeArgs& a, int slots, cudaStream_t st) {
+    using SH = WideShape<CH, MS, 1, ALONE>;
+    auto kern = decode_wide_kernel<CH, MS, 1, ALONE>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SH::smem);
     if (e != cudaSuccess) return e;
     kern<<<slots, SH::W * 32, SH::smem, st>>>(a);
     return cudaGetLastError();
+}
+
+// One block per shot.  `slots`: blocks, no more than the shots or the resident blocks.
+template <int CH, typename MS>
+cudaError_t run_wide(const DecodeArgs& a, int slots, int num_sms, cudaStream_t st) {
+    if constexpr (wide_blocks(CH, (int)sizeof(MS)) == 2)
+        if (slots <= num_sms) return run_wide1<CH, MS, true>(a, slots, st);
+    return run_wide1<CH, MS, false>(a, slots, st);
 }
 
 // Cluster form: the largest number of clusters of CL blocks that can be resident at once

@@ -256,15 +256,16 @@ cudaError_t launch_decode_list_rw(int precision, int list, const DecodeArgs& a, 
 constexpr double kRwMinWeight = 9.5367431640625e-07;  // 2^-20
 // Global-memory tier.  `slots` CTAs each own one scratch slot of global_slot_bytes() for
 // shots of up to max_s defects (a width class's bound); a.gsmax must be the value that
-// function reports.
+// function reports.  Launches of no more slots than SMs run the streaming tier's form of one
+// block per SM (decode_wide.cuh).
 size_t global_slot_bytes(int precision, int max_s, int* gsmax_out);
 // Resident blocks per SM of the global-memory tier for shots of up to max_s defects.
 int global_blocks_per_sm(int precision, int max_s);
-cudaError_t launch_decode_global(int precision, const DecodeArgs& a, int slots,
+cudaError_t launch_decode_global(int precision, const DecodeArgs& a, int slots, int num_sms,
                                  cudaStream_t st);
 // Streaming tier with 16-bit message storage (precision 2 = IEEE half, 3 = bfloat16) for
 // ch columns per lane (kernels_half.cu).
-cudaError_t launch_stream_half(int precision, int ch, const DecodeArgs& a, int slots, cudaStream_t st);
+cudaError_t launch_stream_half(int precision, int ch, const DecodeArgs& a, int slots, int num_sms, cudaStream_t st);
 // Cluster form of the streaming tier (kernels_cluster.cu, kernels_cluster_half.cu): the
 // blocks of a thread-block cluster share one shot and one slot.  stream_cluster_size() is the
 // cluster size a launch of ch columns per lane uses (1: one block per shot) for a requested

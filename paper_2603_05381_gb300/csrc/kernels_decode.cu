@@ -565,7 +565,7 @@ size_t global_slot_bytes(int precision, int max_s, int* gsmax_out) {
     return (size_t)3 * gsmax * gsmax * esz;
 }
 
-cudaError_t launch_decode_global(int precision, const DecodeArgs& a, int slots, cudaStream_t st) {
+cudaError_t launch_decode_global(int precision, const DecodeArgs& a, int slots, int num_sms, cudaStream_t st) {
     if (slots <= 0) return cudaSuccess;
     const int ch = stream_ch(precision, a.gsmax);
     if (ch && 32 * ch == a.gsmax) {
@@ -574,22 +574,22 @@ cudaError_t launch_decode_global(int precision, const DecodeArgs& a, int slots, 
             const int cl = stream_cluster_size(precision, ch, a.stream_cl);
             if (cl > 1) return launch_stream_cluster(precision, ch, cl, a, slots, st);
         }
-        if (precision >= 2) return launch_stream_half(precision, ch, a, slots, st);
+        if (precision >= 2) return launch_stream_half(precision, ch, a, slots, num_sms, st);
         if (precision == 0) {
             if (ch == 8) return run_stream<8>(a, slots, st);
             return run_stream<16>(a, slots, st);
         }
         switch (ch) {
-            case 6: return run_wide<6, float>(a, slots, st);
-            case 8: return run_wide<8, float>(a, slots, st);
-            case 10: return run_wide<10, float>(a, slots, st);
-            case 12: return run_wide<12, float>(a, slots, st);
-            case 14: return run_wide<14, float>(a, slots, st);
-            case 16: return run_wide<16, float>(a, slots, st);
-            case 20: return run_wide<20, float>(a, slots, st);
-            case 24: return run_wide<24, float>(a, slots, st);
-            case 28: return run_wide<28, float>(a, slots, st);
-            default: return run_wide<32, float>(a, slots, st);
+            case 6: return run_wide<6, float>(a, slots, num_sms, st);
+            case 8: return run_wide<8, float>(a, slots, num_sms, st);
+            case 10: return run_wide<10, float>(a, slots, num_sms, st);
+            case 12: return run_wide<12, float>(a, slots, num_sms, st);
+            case 14: return run_wide<14, float>(a, slots, num_sms, st);
+            case 16: return run_wide<16, float>(a, slots, num_sms, st);
+            case 20: return run_wide<20, float>(a, slots, num_sms, st);
+            case 24: return run_wide<24, float>(a, slots, num_sms, st);
+            case 28: return run_wide<28, float>(a, slots, num_sms, st);
+            default: return run_wide<32, float>(a, slots, num_sms, st);
         }
     }
     const size_t smem = global_kernel_smem(a.gsmax);

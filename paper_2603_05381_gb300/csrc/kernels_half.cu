@@ -30,27 +30,27 @@ cudaError_t dispatch_half(int list, const DecodeArgs& a, int num_sms, cudaStream
 }
 
 template <typename MS>
-cudaError_t dispatch_stream_half(int ch, const DecodeArgs& a, int slots, cudaStream_t st) {
+cudaError_t dispatch_stream_half(int ch, const DecodeArgs& a, int slots, int num_sms, cudaStream_t st) {
     switch (ch) {
-        case 6: return run_wide<6, MS>(a, slots, st);
-        case 8: return run_wide<8, MS>(a, slots, st);
-        case 10: return run_wide<10, MS>(a, slots, st);
-        case 12: return run_wide<12, MS>(a, slots, st);
-        case 14: return run_wide<14, MS>(a, slots, st);
-        case 16: return run_wide<16, MS>(a, slots, st);
-        case 20: return run_wide<20, MS>(a, slots, st);
-        case 24: return run_wide<24, MS>(a, slots, st);
-        case 28: return run_wide<28, MS>(a, slots, st);
-        case 32: return run_wide<32, MS>(a, slots, st);
+        case 6: return run_wide<6, MS>(a, slots, num_sms, st);
+        case 8: return run_wide<8, MS>(a, slots, num_sms, st);
+        case 10: return run_wide<10, MS>(a, slots, num_sms, st);
+        case 12: return run_wide<12, MS>(a, slots, num_sms, st);
+        case 14: return run_wide<14, MS>(a, slots, num_sms, st);
+        case 16: return run_wide<16, MS>(a, slots, num_sms, st);
+        case 20: return run_wide<20, MS>(a, slots, num_sms, st);
+        case 24: return run_wide<24, MS>(a, slots, num_sms, st);
+        case 28: return run_wide<28, MS>(a, slots, num_sms, st);
+        case 32: return run_wide<32, MS>(a, slots, num_sms, st);
         default: return cudaErrorInvalidValue;
     }
 }
 
 }  // namespace
 
-cudaError_t launch_stream_half(int precision, int ch, const DecodeArgs& a, int slots, cudaStream_t st) {
-    if (precision == 2) return dispatch_stream_half<__half>(ch, a, slots, st);
-    if (precision == 3) return dispatch_stream_half<__nv_bfloat16>(ch, a, slots, st);
+cudaError_t launch_stream_half(int precision, int ch, const DecodeArgs& a, int slots, int num_sms, cudaStream_t st) {
+    if (precision == 2) return dispatch_stream_half<__half>(ch, a, slots, num_sms, st);
+    if (precision == 3) return dispatch_stream_half<__nv_bfloat16>(ch, a, slots, num_sms, st);
     return cudaErrorInvalidValue;
 }
 

@@ -358,7 +358,7 @@ cudaError_t launch_decode_list_rw(int, int list, const DecodeArgs& a, int, cudaS
         for (int k = 0; k < *a.count; ++k) decode(a, a.list[(int64_t)k * a.list_dir], 0, 1 << 20);
     });
 }
-cudaError_t launch_decode_global(int precision, const DecodeArgs& a, int slots, cudaStream_t st) {
+cudaError_t launch_decode_global(int precision, const DecodeArgs& a, int slots, int, cudaStream_t st) {
     return launch(GLOBAL, a.gsmax, st, [=] {
         // every slot is written before and checked after, as a block that owns it would
         for (int q = 0; q < slots; ++q) ((volatile char*)a.gscratch)[(size_t)q * a.gslot_elems] = (char)q;

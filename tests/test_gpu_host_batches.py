@@ -57,6 +57,28 @@ def test_width_classes_of_a_host_request(torch, case, prec, decoder, forced, ear
             assert [int(x[0]) for x in one] == [int(x[k]) for x in host], (case, s, k)
 
 
+@pytest.mark.parametrize("prec,sizes", [("fp32", (161, 192)), ("fp32", (256,)), ("fp32", (257, 320)), ("fp32", (384,)),
+                                        ("fp32", (448,)), ("fp32", (449, 512)), ("fp16", (193, 256)), ("fp16", (321, 384)),
+                                        ("bf16", (192,)), ("bf16", (384,))])
+@pytest.mark.parametrize("decoder,forced", [("bp4m", "greedy"), ("bp4mf", "greedy"), ("bp4mf", "static")])
+def test_one_block_per_sm_matches_two(torch, prec, sizes, decoder, forced):
+    # a launch of no more shots than SMs has blocks of twice the warps: one shot more, and one alone
+    g, og, _ = _pair(13)
+    n = torch.cuda.get_device_properties(0).multi_processor_count + 1
+    T = 3
+    _, _, synd = _syndromes(torch, og, [sizes[k % len(sizes)] for k in range(n)], seed=45)
+    opts = pkg.make_opts(precision=prec, decoder=decoder, forced=forced, early_exit=False, stream_cluster=1)
+    got = []
+    for k in (n, n - 1, len(sizes)):
+        out = [torch.full((k,), 77, dtype=t, device="cuda") for t in (torch.uint8, torch.uint8, torch.int16)]
+        g.decode_batch(synd[:k], T, opts, *out)
+        torch.cuda.synchronize()
+        got.append([x.cpu().numpy() for x in out])
+    for few in got[1:]:
+        for a, b in zip(got[0], few):
+            assert np.array_equal(a[:len(b)], b)
+
+
 @pytest.mark.parametrize("side", [True, False])
 def test_host_rows_written_by_queued_work(torch, side):
     # a copy into pinned rows, behind a gigabyte of other copies in the caller's stream
