@@ -700,7 +700,9 @@ bool one_width(const GlobalPlan& p, int pio, const bp4m_opts* o, int widest, int
 // items at lists[c], device count and work counter at counts[c] and nexts[c]).  A class of fewer
 // shots than half its resident blocks (typically a few shots above the bulk's width) runs on the
 // second stream beside the others with its own scratch, instead of holding the stream for a
-// whole shot's decode on a few SMs; empty classes are skipped.
+// whole shot's decode on a few SMs; of several such classes the largest stays on `st`, so that the
+// others run beside it and not before or after it (us, FP32, T = 12, one after another -> so: 60 and 160 shots
+// at d = 17 588 -> 358 and 981 -> 827, 20 and 160 at d = 19 521 -> 404 and 1852 -> 1558); empty classes are skipped.
 int launch_global_counted(Workspace& w, const DecodeArgs& a, const GlobalPlan& p, int pio, const bp4m_opts* o,
                           const int32_t* host_cnt, const int32_t* const* lists, const int32_t* counts, int32_t* nexts,
                           int num_sms, cudaStream_t st) {
@@ -711,13 +713,19 @@ int launch_global_counted(Workspace& w, const DecodeArgs& a, const GlobalPlan& p
         CK(cudaEventRecord(w.ev_fork, st));
         CK(cudaStreamWaitEvent(aux, w.ev_fork, 0));
     }
+    int largest = 0, used = 0;
+    for (int c = 0; c < p.gc.n; ++c) {
+        used += host_cnt[c] > 0 ? 1 : 0;
+        if (host_cnt[c] > host_cnt[largest]) largest = c;
+    }
+    if (used < 2) largest = -1;
     cudaError_t e = cudaSuccess;
     // small classes first, so that their few blocks hold their SMs before the large
     // classes' persistent blocks fill the rest
     for (int pass = 0; pass < 2; ++pass)
         for (int c = 0; c < p.gc.n && e == cudaSuccess; ++c) {
             const int cnt = host_cnt[c];
-            const bool small = 2 * cnt < p.full[c];
+            const bool small = c != largest && 2 * cnt < p.full[c];
             if (cnt <= 0 || small != (pass == 0)) continue;
             DecodeArgs b = a;
             b.list = lists[c];

@@ -5,7 +5,7 @@ import ctypes
 import numpy as np
 import pytest
 
-from fake_cuda import CLASSIFY, Fake, build_fake
+from fake_cuda import CLASSIFY, GLOBAL, Fake, build_fake
 from paper_2603_05381_gb300 import _capi
 
 # defect counts: none, every list, and four streaming width classes
@@ -233,3 +233,21 @@ def test_host_counts_small_batches_only(fake, d, n, on_host):
     out = _out(fake, n, "pageable")
     assert fake.decode(g, rows, out) == 0 and _same(fake, rows, out)
     assert (CLASSIFY not in fake.launches()[:, 0]) == on_host
+
+
+@pytest.mark.parametrize("where", ["pageable", "device"])
+def test_small_width_classes_run_beside_the_largest(fake, where):
+    # two shots of one class and one of each of two others, all classes of few shots: the first stays
+    # on the caller's stream, the others share the second
+    lib = fake.lib
+    lib.fake_reset()
+    g = fake.graph()
+    rows = fake.syndromes(g, [300, 170, 250, 310, 410], seed=11)
+    synd = fake.buffer(rows.size, np.uint32, where).reshape(rows.shape)
+    synd[:] = rows
+    out = _out(fake, len(rows), where)
+    st = fake.stream()
+    assert fake.decode(g, synd, out, stream=st) == 0 and _same(fake, rows, out) and lib.fake_list_errors() == 0
+    got = {int(w): int(s) for k, w, s, _ in fake.launches() if k == GLOBAL}
+    assert len(got) == 4 and got[192] == got[256] == got[448] and got[320] != got[192]
+    lib.cudaStreamDestroy(st)
