@@ -527,8 +527,13 @@ int stream_cluster_for(int precision, int gsmax, int requested, int64_t shots, i
     if (precision == 0 || ch == 0 || 32 * ch != gsmax) return 1;
     if (requested != 0) return stream_cluster_size(precision, ch, requested);
     // automatic: one block per shot while the class fills the device at least half; below
-    // that, the size that finishes the class soonest, with the cluster form's measured cost
-    // per shot and SM of about 1.25 + 0.03 CL times one block's
+    // that, the size that finishes the class soonest.  A round of clusters is taken to cost 1.25 + 0.03 CL per
+    // shot and SM, one block per shot 1.  Measured on the present forms (76 shots of one width, T = 12): FP32
+    // 1.2 and 1.0 at clusters of 2 (192 and 256 columns), 1.9, 1.3 and 1.0 at 4 (192, 256, 320), 1.8, 1.6, 1.4 and
+    // 1.2 at 8 (448, 512, 640, 896), 2.3, 2.0, 1.7 and 1.3 at 16; 16-bit messages 1.2 to 1.8 at 4, 1.9 at 8, 1.4
+    // (896) to 2.1 at 16.  Far from it at 320 columns only (76 to 100 shots: 615 us one block per shot, 487 to
+    // 507 in clusters of 4, not taken); a constant that suits these takes 100 shots of 192 columns
+    // from 249 to 324 us.
     if (shots <= 0 || 2 * shots >= full_blocks) return 1;
     double best = 1.0;
     int best_cl = 1;
