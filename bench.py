@@ -42,8 +42,8 @@ KERNEL_OF_REG = {"tier5": "decode_reg_kernel<NB=32, B=4> (s <= 128)",
 # DRAM bytes (read + write) per decoded shot of each FP32 tier kernel, from one ncu capture
 # (dram__bytes_read.sum + dram__bytes_write.sum) of the 65,536-shot case of this workload,
 # divided by the shots the launch decoded; a full launch's traffic is this times its shots.
-DRAM_BYTES_PER_SHOT = {"tier4": 8.536e6 / 10172, "tier5": 12.013e6 / 26656, "tier6": 11.048e6 / 21645,
-                       "tier7": 7.452e6 / 5503}
+DRAM_BYTES_PER_SHOT = {"tier4": 6.256e6 / 10070, "tier5": 9.700e6 / 26803, "tier6": 9.136e6 / 21497,
+                       "tier7": 4.866e6 / 5633}
 # the same with the register-tile form of tiers 5 and 6 (not yet captured for those two)
 DRAM_BYTES_PER_SHOT_REG = {"tier4": DRAM_BYTES_PER_SHOT["tier4"], "tier7": DRAM_BYTES_PER_SHOT["tier7"]}
 METRIC = "decoded shots/s & msg-updates/s vs HBM roofline (d=13 circuit); p50/p99 latency"
