@@ -218,7 +218,6 @@ struct Workspace {
     unsigned char* hb_dev = nullptr;
     unsigned char* hb_pin = nullptr;
     size_t hb_bytes = 0;
-    cudaEvent_t ev_in = nullptr;  // the work queued before the call (decode_host)
     // B-BP4MF first stage
     int64_t qcap = 0;
     uint8_t* qconv = nullptr;
@@ -252,6 +251,7 @@ struct bp4m_graph {
     bool prepared[4] = {false, false, false, false};
     Workspace ws;
     ListLanes lanes;  // of this graph's calls and its derived graphs'
+    cudaEvent_t ev_in = nullptr;  // the work queued before a call (decode_host)
     bp4m_graph() { ws.lanes = &lanes; }
     // measurement: event pairs around every launch while profiling is on
     struct ProfEvent {
@@ -451,6 +451,7 @@ int ensure_uploaded(bp4m_graph* g) {
             CK(cudaMemcpy(g->rw_adj[ty], ent.data(), ent.size() * 4, cudaMemcpyHostToDevice));
         }
     }
+    if (!g->ev_in) CK(cudaEventCreateWithFlags(&g->ev_in, cudaEventDisableTiming));
     g->uploaded = true;
     return BP4M_OK;
 }
@@ -474,7 +475,6 @@ void free_ws(Workspace& w) {
     cudaFreeHost(w.host_small);
     cudaFreeHost(w.host_ctr);
     if (w.ev_small) cudaEventDestroy(w.ev_small);
-    if (w.ev_in) cudaEventDestroy(w.ev_in);
     cudaFree(w.hb_dev);
     cudaFreeHost(w.hb_pin);
     cudaFree(w.qconv);
@@ -928,10 +928,10 @@ int decode_host(bp4m_graph* g, Workspace& w, int ty, const uint32_t* synd, int64
     // The host reads the rows here, where a copy in the stream would have followed the work queued
     // before the call (it may still be writing them: pinned rows, or any host memory that the GPU
     // writes).  An event rather than a wait for the stream: in the legacy stream, or a blocking one,
-    // it also follows the work of the streams that those wait for.  1.2 us where nothing is queued.
-    if (!w.ev_in) CK(cudaEventCreateWithFlags(&w.ev_in, cudaEventDisableTiming));
-    CK(cudaEventRecord(w.ev_in, st));
-    CK(cudaEventSynchronize(w.ev_in));
+    // it also follows the work of the streams that those wait for.  Two of a d = 5 shot's 42 us where nothing
+    // is queued (a wait for the stream, or asking it, takes as long).
+    CK(cudaEventRecord(g->ev_in, st));
+    CK(cudaEventSynchronize(g->ev_in));
     std::memset(hp + L.ctr, 0, L.items - L.ctr);
     std::memcpy(hp + L.synd, synd, (size_t)shots * nw * sizeof(uint32_t));
     // defect counts, lists by counting
@@ -2536,6 +2536,7 @@ void bp4m_free_graph(bp4m_graph* g) {
         }
         free_ws(g->ws);
     }
+    if (g->ev_in) cudaEventDestroy(g->ev_in);
     g->lanes.free();  // (derived graphs may have used them where this one was not uploaded)
     delete g;
 }
