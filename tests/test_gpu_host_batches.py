@@ -79,9 +79,9 @@ def test_one_block_per_sm_matches_two(torch, prec, sizes, decoder, forced):
             assert np.array_equal(a[:len(b)], b)
 
 
-@pytest.mark.parametrize("side", [True, False])
-def test_host_rows_written_by_queued_work(torch, side):
-    # a copy into pinned rows, behind a gigabyte of other copies in the caller's stream
+@pytest.mark.parametrize("prio", [None, 0, -1])  # the default stream, side streams of two priorities
+def test_host_rows_written_by_queued_work(torch, prio):
+    # a copy into pinned rows, behind gigabytes of other copies in the caller's stream
     g, og, _ = _pair(9)
     n, T = 64, 10
     _, packed, synd = _syndromes(torch, og, [1 + k % 40 for k in range(n)], seed=43)
@@ -92,7 +92,7 @@ def test_host_rows_written_by_queued_work(torch, side):
     a = torch.zeros(1 << 28, dtype=torch.float32, device="cuda")
     b = torch.empty_like(a)
     torch.cuda.synchronize()
-    st = torch.cuda.Stream() if side else torch.cuda.default_stream()
+    st = torch.cuda.default_stream() if prio is None else torch.cuda.Stream(priority=prio)
     got = [np.full(n, 77, dtype=t) for t in (np.uint8, np.uint8, np.int16)]
     with torch.cuda.stream(st):
         for _ in range(20):
